@@ -223,7 +223,10 @@ enum {
 /* Copy an internal buffer to host memory as doubles, without K padding:
  * PHI/MICRO_F/RES/DPHI [2][N][K], FACE [2][F][K], FSTATE [F][16], W/Q/MACRO_F/WT
  * [N][6], DT [N][3] (CFL step, implicit step, eps^2), S [F], TAUT [N].
- * `count` is the number of doubles the caller's buffer holds. */
+ * `count` is the number of doubles the caller's buffer holds.  FACE, FSTATE and
+ * MICRO_F are those of the last iteration or step; after rk_surface, rk_aero or, in
+ * RK_MIXED contexts, the adjoint's products they are those of the present state,
+ * evaluated when they are first read. */
 int rk_debug_get(rk_ctx* ctx, int which, double* host_out, int64_t count);
 /* Selected rows of a distribution-shaped verification buffer, for checks of large
  * cases one cell or face at a time: which = RK_BUF_PHI, RK_BUF_RES, RK_BUF_DPHI,

@@ -292,12 +292,12 @@ static cudaError_t adj_prepare_t(rk_ctx* ctx, AdjState& A) {
     d.iterp = A.iterp;
     if constexpr (sizeof(S) == 4) {
         // the context's own FP32 reconstruction, written to its face array (scratch of the
-        // iteration)
+        // iteration: the rows are no finished faces afterwards)
         rk::Dev<float> df = ctx->df;
         df.iterp = A.iterp;
         cudaError_t e = rk::Launch<float>::recon(df, s, ctx->prof);
         if (e != cudaSuccess) return e;
-        ctx->faces_partial = false;
+        ctx->faces_partial = ctx->faces_redo = true;
     } else {
         d.face = A.f0;
         rk::launch_recon_d<false>(d, s, nullptr, (int)ctx->N);

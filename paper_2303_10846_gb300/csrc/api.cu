@@ -379,7 +379,7 @@ static int bind_impl(rk_ctx* ctx, rk::Dev<T>& d) {
     std::sort(wall_cell.begin(), wall_cell.end());
     wall_cell.erase(std::unique(wall_cell.begin(), wall_cell.end()), wall_cell.end());
     ctx->n_wall_cell = (int)wall_cell.size();
-    ctx->faces_partial = false;
+    ctx->faces_partial = ctx->faces_redo = false;
     CK(h2d(d.vol, ctx->cv.data(), N * 8));
     CK(h2d(d.cx, cxs.data(), 3 * N * 8));
     CK(h2d(d.colour, ctx->col.data(), N * 4));
@@ -607,7 +607,9 @@ static cudaError_t launch_step(rk_ctx* ctx, rk::Dev<T>& d, int step, cudaStream_
 // there to be read, and verification calls that follow (complete_faces) get every face.
 template <typename T>
 static cudaError_t wall_faces(rk_ctx* ctx, rk::Dev<T>& d) {
+    ctx->faces_redo = true;
     if (ctx->debug) {
+        ctx->faces_partial = false;
         cudaError_t e = launch_step(ctx, d, RK_STEP_RECON, ctx->stream);
         return e != cudaSuccess ? e : rk::Launch<T>::faces(d, ctx->stream, ctx->prof);
     }
@@ -626,8 +628,12 @@ static cudaError_t complete_faces(rk_ctx* ctx, rk::Dev<T>& d) {
 template <typename T>
 static int step_impl(rk_ctx* ctx, rk::Dev<T>& d, int step) {
     if (step < RK_STEP_RECON || step > RK_STEP_MICRO) return fail(ctx, RK_EINVAL, "rk_step: unknown step");
-    if (step == RK_STEP_FACES || step == RK_STEP_FLUXES) CK(complete_faces(ctx, d));
-    if (step == RK_STEP_RECON) ctx->faces_partial = false;
+    // after a wall or adjoint call in between: the face step starts from the reconstruction;
+    // the fluxes, and the verification reads after the state has moved on (MICRO), take the
+    // finished faces of the state of that call
+    if (step == RK_STEP_FACES && ctx->faces_redo) CK(launch_step(ctx, d, RK_STEP_RECON, ctx->stream));
+    if (step == RK_STEP_RECON || step == RK_STEP_FACES) ctx->faces_partial = ctx->faces_redo = false;
+    if (step == RK_STEP_FLUXES || step == RK_STEP_MICRO) CK(complete_faces(ctx, d));
     cudaError_t e = launch_step(ctx, d, step, ctx->stream);
     if (e != cudaSuccess) return fail(ctx, RK_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
     if (step == RK_STEP_MICRO) ctx->iter++;
@@ -707,7 +713,7 @@ static int iteration(rk_ctx* ctx, rk::Dev<T>& d) {
             ctx->use_graph = false;
             (void)cudaGetLastError();
         } else {
-            ctx->faces_partial = false;
+            ctx->faces_partial = ctx->faces_redo = false;
             CK(cudaGraphLaunch(ctx->gexec, ctx->stream));
             ctx->prof.launches += ctx->graph_kernels;
             ctx->iter++;

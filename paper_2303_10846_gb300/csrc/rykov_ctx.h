@@ -75,9 +75,12 @@ struct rk_ctx {
     int* wall_b_dev = nullptr;
     int* wall_cell_dev = nullptr;                     // cells with a wall face
     int n_wall_cell = 0;
-    // the face arrays hold the present state at the wall faces only (rk_surface, rk_aero):
-    // completed when a verification call reads them
-    bool faces_partial = false;
+    // Face rows after a call that uses the face array as scratch (rk_surface, rk_aero, the
+    // FP32 adjoint).  faces_partial: they are not the finished rows of the present state
+    // (wall faces only, or the bare reconstruction) and are completed before anything reads
+    // them.  faces_redo: the face step works in place on the reconstruction, so it has to
+    // reconstruct first.
+    bool faces_partial = false, faces_redo = false;
     void* dbg = nullptr;                              // [2][N][Kp] T (debug contexts)
     double* pin = nullptr;                            // pinned host: 16 doubles
     int64_t iter = 0;
