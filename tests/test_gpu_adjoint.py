@@ -294,3 +294,33 @@ def test_adjoint_sphere_converges_and_matches_finite_differences(sphere_first_or
         for idx in (0, 1, 2, 5):
             assert abs(g[idx] - fd[o][idx]) <= 1e-6 * scale, (o, idx, g[idx], fd[o][idx])
     m.close()
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_adjoint_solve_depends_on_the_present_state_alone(prec):
+    """put_state and a bounded solve on a context that never iterated, its workspace full of
+    NaN before the bind, and on one that iterated elsewhere: the same bits."""
+    from paper_2303_10846_gb300.rykov import _ptr
+    wl = tet()
+    donor = _solver_prec(wl, prec, 4)
+    donor.iterate(4)
+    x = donor.get_state()
+    out = []
+    for fresh in (True, False):
+        s = _solver_prec(wl, prec, 4)
+        if fresh:
+            s.workspace.fill_(255)
+            s._check(s.L.rk_bind_workspace(s.h, _ptr(s.workspace), s.workspace.numel()))
+            s.bind_adjoint(4)
+        else:
+            prim = wl.prim0.copy()
+            prim[:, 0] *= 2.0
+            prim[:, 4:6] *= 3.0
+            s.set_state_prim(prim)
+            s.iterate(3)
+        s.put_state(x)
+        it, rel, J, dJdp = s.adjoint_solve("heat", max_iter=6, tol=1e-14)
+        assert it == 6 and np.isfinite(rel)
+        out.append((s.adjoint_get(), np.array([rel, J]), dJdp))
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
