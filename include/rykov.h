@@ -340,7 +340,8 @@ const char* rk_noalloc_last_error(void);
  *       solution of the same objective at the same state (0 otherwise).  Returns the
  *       iterations done, the final relative residual (recomputed, not estimated),
  *       J, and the total derivative dJdp[6] = dJ/dp + lam^T dR/dp.  RK_EDIVERGED if
- *       the residual becomes non-finite.
+ *       the residual becomes non-finite.  The macro operator's spectral radii are the
+ *       last iteration's, or those of W where there was none since rk_set_state(_prim).
  *   rk_adjoint_get(ctx, lam, on_device): the last adjoint solution (packed). */
 /* Fused multiply-add throughput of the current device (a measurement utility with
  * no counterpart in the paper): the ALU ceiling of the FP64 form, whose per-velocity

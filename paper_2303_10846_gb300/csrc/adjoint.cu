@@ -395,9 +395,11 @@ static cudaError_t adj_apply(rk_ctx* ctx, AdjState& A, const double* v, double* 
                          : adj_apply_t<double>(ctx, A, v, o, obj_scale, objective, false, o, ctx->Kp);
 }
 
-// What the preconditioner needs of the state: the inverse micro diagonal, the spectral radii
-// of W (those in memory are the last iteration's, of another state, or none at all) and the
-// constants of the transposed macro updates.  Once per solve.
+// What the preconditioner needs of the state: the inverse micro diagonal and the constants
+// of the transposed macro updates.  Once per solve.  Its spectral radii are the last
+// iteration's, one step behind the state of a march, or W's where no iteration has formed
+// any since a state was set (they enter the preconditioner alone, so a solve that reaches
+// its tolerance does not depend on them; one that stops at max_iter does).
 template <typename S>
 static cudaError_t adj_pc_prepare_t(rk_ctx* ctx, AdjState& A) {
     const rk::Dev<double> d = dview(ctx, A);
@@ -405,9 +407,12 @@ static cudaError_t adj_pc_prepare_t(rk_ctx* ctx, AdjState& A) {
     const rk::AdjArr<S> r = adj_arr<S>(ctx, A, d, A.vzero, A.tmp);
     constexpr int W = rk::ADJ_WPB;
     rk::k_adj_sweep<W, S, true><<<rk::cdv(ctx->N, W), W * 32, 0, ctx->stream>>>(d, a, r, nullptr, (int)ctx->N, nullptr, nullptr);
-    rk::k_face_radius<double><<<rk::cdv(ctx->F, 64), 64, 0, ctx->stream>>>(d);
+    if (!ctx->have_radii) {
+        rk::k_face_radius<double><<<rk::cdv(ctx->F, 64), 64, 0, ctx->stream>>>(d);
+        A.launches++;
+    }
     rk::k_adj_macro_prep<<<rk::cdv(ctx->N, 128), 128, 0, ctx->stream>>>(d, ctx->sched.col_cell, A.tau, A.mC, A.mS);
-    A.launches += 3;
+    A.launches += 2;
     return cudaGetLastError();
 }
 static cudaError_t adj_pc_prepare(rk_ctx* ctx, AdjState& A) {

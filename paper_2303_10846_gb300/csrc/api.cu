@@ -483,7 +483,7 @@ static int bind_impl(rk_ctx* ctx, rk::Dev<T>& d) {
     if (e != cudaSuccess) return fail(ctx, RK_ECUDA, std::string("setup kernels: ") + cudaGetErrorString(e));
     CK(cudaStreamSynchronize(s));
     ctx->bound = true;
-    ctx->have_state = false;
+    ctx->have_state = ctx->have_radii = false;
     ctx->bind_gen++;
     return RK_OK;
 }
@@ -526,6 +526,7 @@ static int set_state_prim_impl(rk_ctx* ctx, rk::Dev<T>& d, const double* prim, c
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->iter = 0;
     ctx->have_state = true;
+    ctx->have_radii = false;
     ctx->state_ver++;
     return RK_OK;
 }
@@ -562,6 +563,7 @@ extern "C" int rk_set_state(rk_ctx* ctx, const double* W, const double* q, const
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->iter = 0;
     ctx->have_state = true;
+    ctx->have_radii = false;
     ctx->state_ver++;
     return RK_OK;
 }
@@ -636,6 +638,7 @@ static int step_impl(rk_ctx* ctx, rk::Dev<T>& d, int step) {
     if (step == RK_STEP_FLUXES || step == RK_STEP_MICRO) CK(complete_faces(ctx, d));
     cudaError_t e = launch_step(ctx, d, step, ctx->stream);
     if (e != cudaSuccess) return fail(ctx, RK_ECUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
+    if (step == RK_STEP_FLUXES) ctx->have_radii = true;
     if (step == RK_STEP_MICRO) ctx->iter++;
     ctx->state_ver++;
     return RK_OK;
@@ -714,6 +717,7 @@ static int iteration(rk_ctx* ctx, rk::Dev<T>& d) {
             (void)cudaGetLastError();
         } else {
             ctx->faces_partial = ctx->faces_redo = false;
+            ctx->have_radii = true;
             CK(cudaGraphLaunch(ctx->gexec, ctx->stream));
             ctx->prof.launches += ctx->graph_kernels;
             ctx->iter++;

@@ -81,6 +81,9 @@ struct rk_ctx {
     // them.  faces_redo: the face step works in place on the reconstruction, so it has to
     // reconstruct first.
     bool faces_partial = false, faces_redo = false;
+    // an iteration (or the flux step) has formed the spectral radii since the workspace was
+    // bound or a state was set by rk_set_state(_prim)
+    bool have_radii = false;
     void* dbg = nullptr;                              // [2][N][Kp] T (debug contexts)
     double* pin = nullptr;                            // pinned host: 16 doubles
     int64_t iter = 0;

