@@ -696,6 +696,13 @@ __global__ void __launch_bounds__(WPB * 32) k_adj_face_b(Dev<double> c, AdjBufs 
     }
 }
 
+// u.n > 0 as the reconstruction of the same arithmetic decides it
+template <typename S>
+__device__ __forceinline__ bool adj_outflow(const VelF& u, float4 n, S ux, S uy, S uz, const Q4<S>& N) {
+    if constexpr (sizeof(S) == 8) return outflow(u, n, ux, uy, uz, N.x, N.y, N.z);
+    else return dot_rn(ux, uy, uz, N.x, N.y, N.z) > S(0);
+}
+
 // ------------------------------------------------------------------------------------
 // boundary faces: reverse of the wall / farfield treatment (no interface collision).
 // Seeds: -A (u.n) v_i / V_i from R_phi, plus obj_scale times the derivative of the
@@ -721,6 +728,13 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
     const float4 nf = make_float4((float)nx, (float)ny, (float)nz, 0.f);
     const double* bv = c.bcv + 5 * bc;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    // the upwind decision of the reconstruction and of the gather, on their values of u and n:
+    // f0 holds, and the gather reads, the velocities that leave the cell by that decision
+    auto leaves = [&](int k) {
+        VelF uf{};
+        if constexpr (sizeof(S) == 8) uf = vel_f(c, k);
+        return adj_outflow(uf, nf, r.u[k], r.u[c.Kp + k], r.u[2 * c.Kp + k], Q4<S>{(S)nx, (S)ny, (S)nz, S(0)});
+    };
     if (threadIdx.x == 0) {
         const double T = bv[4], RT = c.R * T, an = 2.0 * PI * RT;
         mc[0] = (wall ? 1.0 : bv[0]) / (an * sqrt(an));
@@ -761,7 +775,7 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
         for (int k = threadIdx.x; k < c.K; k += BS) {
             const double ux = c.u[k], uy = c.u[c.Kp + k], uz = c.u[2 * c.Kp + k];
             const double wu = c.w[k] * (ux * nx + uy * ny + uz * nz);
-            if (outflow(vel_f(c, k), nf, ux, uy, uz, nx, ny, nz)) {
+            if (leaves(k)) {
                 v[0] += wu * (double)g0[k];
             } else {
                 double cx, cy, cz, c2;
@@ -793,7 +807,7 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
             }
         }
         double gf = 0.0, hf = 0.0;
-        if (outflow(vel_f(c, k), nf, ux, uy, uz, nx, ny, nz)) {
+        if (leaves(k)) {
             if (seed != 0.0) {               // J and the force: of the objective only
                 gf = (double)g0[k];
                 hf = (double)h0[k];
@@ -844,7 +858,7 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
         const double numb = sh[0] / dn;
         for (int k = threadIdx.x; k < c.K; k += BS) {
             const double ux = c.u[k], uy = c.u[c.Kp + k], uz = c.u[2 * c.Kp + k];
-            if (outflow(vel_f(c, k), nf, ux, uy, uz, nx, ny, nz))
+            if (leaves(k))
                 gbar[k] = (S)((double)gbar[k] + numb * (c.w[k] * (ux * nx + uy * ny + uz * nz)));
         }
     }
@@ -881,11 +895,6 @@ template <typename S>
 __device__ __forceinline__ S adj_quot(S a, S b) {
     if constexpr (sizeof(S) == 8) return quot(a, b);
     else return lim_div(a, b);
-}
-template <typename S>
-__device__ __forceinline__ bool adj_outflow(const VelF& u, float4 n, S ux, S uy, S uz, const Q4<S>& N) {
-    if constexpr (sizeof(S) == 8) return outflow(u, n, ux, uy, uz, N.x, N.y, N.z);
-    else return dot_rn(ux, uy, uz, N.x, N.y, N.z) > S(0);
 }
 template <int WPB, typename S, int MS>
 __global__ void __launch_bounds__(WPB * 32) k_adj_gather(Dev<double> c, AdjBufs a, AdjArr<S> r) {

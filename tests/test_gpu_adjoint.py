@@ -326,3 +326,39 @@ def test_adjoint_solve_without_an_iteration_before_it(prec):
         out.append((s.adjoint_get(), np.array([rel, J]), dJdp))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+def test_mixed_adjoint_at_grazing_velocities(monkeypatch):
+    """Velocities along a wall face whose u.n rounds to a positive number in FP32 and is not
+    positive in FP64 (and the other way round): the boundary kernel and the gather have to
+    take the same side, or the gather reads what an earlier call left in its scratch."""
+    wl = TW.tiny_tet(n_gh=4, lim=2, cfl_imp=20.0)
+    m, rng = wl.mesh, np.random.default_rng(2)
+    wall = np.nonzero(m.face_cell[:, 1] == -1)[0]
+    f32 = np.float32
+    extra, kinds = [], set()
+    for f in wall:
+        n = m.face_normal[f]
+        for _ in range(4):
+            u = np.cross(n, rng.normal(size=3))
+            d64 = (u[0] * n[0] + u[1] * n[1]) + u[2] * n[2]
+            a, b = u.astype(f32), n.astype(f32)
+            d32 = f32(f32(a[0] * b[0]) + f32(a[1] * b[1])) + f32(a[2] * b[2])
+            if (d64 > 0) != (d32 > 0):
+                extra.append(u)
+                kinds.add(bool(d32 > 0))
+    assert len(kinds) == 2
+    wl.dvs = I.DVS(u=np.concatenate([wl.dvs.u, extra]),
+                   w=np.concatenate([wl.dvs.w, np.full(len(extra), 1e-3 * wl.dvs.w.mean())]))
+    s = _solver_prec(wl, "mixed", 2)
+    s.iterate(2)
+    v = rng.standard_normal(s.state_len)
+    out, pp = s.vjp(v)
+    s.steady_residual()                           # fills the scratch with FP64 face values
+    again, pp2 = s.vjp(v)
+    assert np.isfinite(out).all() and np.array_equal(out, again) and np.array_equal(pp, pp2)
+    monkeypatch.setenv("RYKOV_ADJ_FP64", "1")
+    out64, _ = s.vjp(v)
+    st = Steady(wl)
+    for a, b in zip(_blocks(st, out), _blocks(st, out64)):
+        assert _rel(a, b) < 1e-5
