@@ -339,13 +339,15 @@ static void adj_gather(const rk::Dev<double>& d, const rk::AdjBufs& a, const rk:
 
 // o = (dR/dX)^T v (padded vectors), pout = (dR/dp)^T v.  v null: v = 0, for which only the
 // boundary faces' seeds and the gathers are run: with obj_scale = 1 that gives dJ/dX,
-// pout[0-5] = dJ/dp|_X, pout[6] = J, pout[7-9] = force.  have_vf: A.vf holds the phi block
-// of v already.  dst, ld: where the phi block of the result goes (rows of ld doubles).
+// pout[0-5] = dJ/dp|_X, pout[6] = J, pout[7-9] = force.  src: A.vf holds the phi block
+// of v already, whose FP64 phi block is then that of src (the packed vector), which may be
+// dst: the last kernel alone writes there.  dst, ld: where the phi block of the result goes
+// (rows of ld doubles).
 template <typename S>
 static cudaError_t adj_apply_t(rk_ctx* ctx, AdjState& A, const double* v, double* o, double obj_scale, int objective,
-                               bool have_vf, double* dst, int ld) {
+                               const double* src, double* dst, int ld) {
     constexpr int W = rk::ADJ_WPB;
-    const bool zero = v == nullptr;
+    const bool zero = v == nullptr, have_vf = src != nullptr;
     if (zero) v = A.vzero;
     const size_t N = ctx->N, NK2 = 2 * N * (size_t)ctx->Kp;
     rk::AdjBufs a = adj_bufs(ctx, A, v, o);
@@ -379,7 +381,7 @@ static cudaError_t adj_apply_t(rk_ctx* ctx, AdjState& A, const double* v, double
         }
     }
     if (ctx->Fb) {
-        rk::k_adj_face_boundary<128, S><<<ctx->Fb, 128, 0, s>>>(d, a, r);
+        rk::k_adj_face_boundary<128, S><<<ctx->Fb, 128, 0, s>>>(d, a, r, have_vf ? src : v, have_vf ? (int)ctx->K : ctx->Kp);
         rk::k_adj_params<<<1, 320, 0, s>>>(A.fpar, ctx->Fb, A.pout);
         A.launches += 2;
     } else if ((e = cudaMemsetAsync(A.pout, 0, 16 * sizeof(double), s)) != cudaSuccess) {
@@ -391,8 +393,8 @@ static cudaError_t adj_apply_t(rk_ctx* ctx, AdjState& A, const double* v, double
     return cudaGetLastError();
 }
 static cudaError_t adj_apply(rk_ctx* ctx, AdjState& A, const double* v, double* o, double obj_scale, int objective) {
-    return adj_fp32(ctx) ? adj_apply_t<float>(ctx, A, v, o, obj_scale, objective, false, o, ctx->Kp)
-                         : adj_apply_t<double>(ctx, A, v, o, obj_scale, objective, false, o, ctx->Kp);
+    return adj_fp32(ctx) ? adj_apply_t<float>(ctx, A, v, o, obj_scale, objective, nullptr, o, ctx->Kp)
+                         : adj_apply_t<double>(ctx, A, v, o, obj_scale, objective, nullptr, o, ctx->Kp);
 }
 
 // What the preconditioner needs of the state: the inverse micro diagonal and the constants
@@ -654,11 +656,11 @@ extern "C" int rk_vjp(rk_ctx* ctx, const double* v, double* out, double* out_par
     if (adj_fp32(ctx)) {
         CK(adj_unpack(ctx, A, src, A.vf, A.rv));
         CK(adj_prepare(ctx, A));
-        CK(adj_apply_t<float>(ctx, A, A.rv, A.tmp, 0.0, 0, true, to, (int)ctx->K));
+        CK(adj_apply_t<float>(ctx, A, A.rv, A.tmp, 0.0, 0, src, to, (int)ctx->K));
     } else {
         CK(adj_unpack(ctx, A, src, A.rv, A.rv));
         CK(adj_prepare(ctx, A));
-        CK(adj_apply_t<double>(ctx, A, A.rv, A.tmp, 0.0, 0, true, to, (int)ctx->K));
+        CK(adj_apply_t<double>(ctx, A, A.rv, A.tmp, 0.0, 0, nullptr, to, (int)ctx->K));
     }
     CK(adj_pack(ctx, A, (const double*)nullptr, A.tmp + n1, A.tmp + n1 + 6 * N, to));
     if (out_params) CK(cudaMemcpyAsync(A.hpin, A.pout, 6 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));

@@ -708,10 +708,13 @@ __device__ __forceinline__ bool adj_outflow(const VelF& u, float4 n, S ux, S uy,
 // Seeds: -A (u.n) v_i / V_i from R_phi, plus obj_scale times the derivative of the
 // objective at wall faces (heat: A w (u.n)(|u|^2/2 g + h); drag: A w (u.n)(u.e) g).
 // Writes fbar at outgoing velocities and per face fpar = (dT_w, drho_inf, dU_inf[3],
-// dT_inf, J_f, force_f[3]).  One block per boundary face, FP64 arithmetic.
+// dT_inf, J_f, force_f[3]).  One block per boundary face, FP64 arithmetic on the FP64 vector
+// (v: its phi block, rows of ldv doubles), in FP32 contexts too: (dR/dp)^T v comes from here
+// alone, and fbar is rounded once, when it is stored.
 // ------------------------------------------------------------------------------------
 template <int BS, typename S>
-__global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs a, AdjArr<S> r) {
+__global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs a, AdjArr<S> r, const double* v,
+                                                          int ldv) {
     constexpr int NW = BS / 32;
     __shared__ double red[NW][6], sh[8], mc[8];
     const int b = blockIdx.x;
@@ -719,7 +722,7 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
     const int bc = -1 - c.fc[2 * f + 1];
     const int i = c.fc[2 * f];
     const bool wall = c.bck[bc] == 0;
-    const size_t FK = (size_t)c.F * c.Kp, NK = (size_t)c.N * c.Kp;
+    const size_t FK = (size_t)c.F * c.Kp;
     const S* g0 = r.f0 + (size_t)f * c.Kp;
     const S* h0 = g0 + FK;
     S* gbar = r.fbar + (size_t)f * c.Kp;
@@ -747,7 +750,14 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
     }
     __syncthreads();
     const double RT = mc[4], sv = mc[5], seed = wall ? a.obj_scale : 0.0;
-    const S* vg = r.v + (size_t)i * c.Kp;
+    const double *vg = v + (size_t)i * ldv, *vh = vg + (size_t)c.N * ldv;
+    // adjoint of g_ij at velocity k: -A (u.n) v / V and the objective's seed
+    auto g_seed = [&](int k, double un, double wu, double u2h, double ux, double uy, double uz) {
+        double x = sv * un * vg[k];
+        if (seed != 0.0)
+            x += seed * A * wu * (a.objective == 0 ? u2h : ux * a.edrag[0] + uy * a.edrag[1] + uz * a.edrag[2]);
+        return x;
+    };
     // |c|^2 and M at velocity k
     auto maxw = [&](int k, double& cx, double& cy, double& cz, double& c2) {
         cx = c.u[k] - bv[1];
@@ -796,23 +806,16 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
         const double ux = c.u[k], uy = c.u[c.Kp + k], uz = c.u[2 * c.Kp + k], w = c.w[k];
         const double un = ux * nx + uy * ny + uz * nz, wu = w * un;
         const double u2h = 0.5 * (ux * ux + uy * uy + uz * uz);
-        double wgb = sv * un * (double)vg[k], whb = sv * un * (double)vg[NK + k];
-        if (seed != 0.0) {
-            const double sw = seed * A * wu;
-            if (a.objective == 0) {
-                wgb += sw * u2h;
-                whb += sw;
-            } else {
-                wgb += sw * (ux * a.edrag[0] + uy * a.edrag[1] + uz * a.edrag[2]);
-            }
-        }
+        const double wgb = g_seed(k, un, wu, u2h, ux, uy, uz);
+        double whb = sv * un * vh[k];
+        if (seed != 0.0 && a.objective == 0) whb += seed * A * wu;
         double gf = 0.0, hf = 0.0;
         if (leaves(k)) {
             if (seed != 0.0) {               // J and the force: of the objective only
                 gf = (double)g0[k];
                 hf = (double)h0[k];
             }
-            gbar[k] = (S)wgb;
+            if (!wall) gbar[k] = (S)wgb;     // (walls: below, with the share through rho_w)
             hbar[k] = (S)whb;
         } else {
             double cx, cy, cz, c2;
@@ -858,8 +861,10 @@ __global__ void __launch_bounds__(BS) k_adj_face_boundary(Dev<double> c, AdjBufs
         const double numb = sh[0] / dn;
         for (int k = threadIdx.x; k < c.K; k += BS) {
             const double ux = c.u[k], uy = c.u[c.Kp + k], uz = c.u[2 * c.Kp + k];
-            if (leaves(k))
-                gbar[k] = (S)((double)gbar[k] + numb * (c.w[k] * (ux * nx + uy * ny + uz * nz)));
+            if (leaves(k)) {
+                const double un = ux * nx + uy * ny + uz * nz, wu = c.w[k] * un;
+                gbar[k] = (S)(g_seed(k, un, wu, 0.5 * (ux * ux + uy * uy + uz * uz), ux, uy, uz) + numb * wu);
+            }
         }
     }
 }

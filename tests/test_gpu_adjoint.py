@@ -362,3 +362,26 @@ def test_mixed_adjoint_at_grazing_velocities(monkeypatch):
     st = Steady(wl)
     for a, b in zip(_blocks(st, out), _blocks(st, out64)):
         assert _rel(a, b) < 1e-5
+
+
+def test_mixed_boundary_terms_are_fp64_and_rounded_once(monkeypatch):
+    """First order, so that the face values are the state's in both arithmetics: (dR/dp)^T v
+    comes from the boundary kernel alone, FP64 on the FP64 vector (1e-12: the order of the
+    operations); dJ/dphi of a cell with one wall face is that face's adjoint, rounded to
+    FP32 once (2^-24 of every entry)."""
+    wl = TW.tiny_tet(n_gh=5, lim=2, cfl_imp=20.0)
+    s = _solver_prec(wl, "mixed", 2)
+    s.iterate(3)
+    v = np.random.default_rng(6).standard_normal(s.state_len)
+    _, pp = s.vjp(v)
+    _, g, dp = s.objective("heat")
+    monkeypatch.setenv("RYKOV_ADJ_FP64", "1")
+    _, pp64 = s.vjp(v)
+    _, g64, dp64 = s.objective("heat")
+    assert np.abs(pp - pp64).max() <= 1e-12 * np.abs(pp64).max()
+    assert np.abs(dp - dp64).max() <= 1e-12 * np.abs(dp64).max()
+    fc = wl.mesh.face_cell
+    one = np.bincount(fc[fc[:, 1] == -1, 0], minlength=s.N) == 1
+    a, b = (x[:2 * s.N * s.K].reshape(2, s.N, s.K)[:, one] for x in (g, g64))
+    assert one.sum() > 10 and np.abs(b).max() > 0
+    assert (np.abs(a - b) <= 2.0 ** -24 * (1 + 1e-6) * np.abs(b)).all()
