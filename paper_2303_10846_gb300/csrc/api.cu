@@ -309,7 +309,7 @@ static size_t carve(rk_ctx* ctx, char* base, rk::Dev<T>& d) {
     d.cellres = cv.take<double>(12 * N); d.res12 = cv.take<double>(16);
     d.ms = 0;
     for (size_t i = 0; i < N; ++i) d.ms = std::max(d.ms, ctx->slot_off[i + 1] - ctx->slot_off[i]);
-    d.mPc = cv.take<double>(8 * N); d.mCon = cv.take<double>(16 * N);
+    d.mPc = cv.take<double>(8 * N); d.mDw = cv.take<double>(rk::MACRO_INC<T> ? 8 * N : 0); d.mCon = cv.take<double>(16 * N);
     d.mSlot = cv.take<double>(4 * N * d.ms);
     d.cell_pos = cv.take<int>(N); d.mNbr = cv.take<int>(N * d.ms);
     d.bar = cv.take<unsigned int>(4);

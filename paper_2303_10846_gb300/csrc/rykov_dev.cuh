@@ -114,10 +114,10 @@ struct DevBase {
         *cellres, *res12;
     // macro PR-SGS work, by colour position (cells in col_cell order, so that the cells of
     // one phase are contiguous and a point update needs no index but its own): the
-    // current iterate [N][8], the constants of a point update [15][N], and for each of a
+    // current iterate [N][8] and its increments [N][8], the constants of a point update [15][N], and for each of a
     // cell's ms face slots the scaled normal with the spectral coefficient [4][ms][N] and
     // the neighbour's position (-1: boundary or no face) [ms][N]; see macro_point
-    double *mPc, *mCon, *mSlot;
+    double *mPc, *mDw, *mCon, *mSlot;
     const int *cell_pos, *mNbr;
     int ms;                              // most faces of one cell
     unsigned int* bar;                   // grid-barrier state of the cooperative macro solve
@@ -1363,32 +1363,46 @@ __global__ void k_iter_begin(Dev<T> c) {
 // Macro PR-SGS (Eq. implicit_mac_equ_fin)
 // ------------------------------------------------------------------------------------
 // Point update of cell i with the current iterate W~_j = W_j + dW~_j of its neighbours,
-//   dW~_i = [-F_i - sum_j (A/2V) ((G(W~_j) - G(W_j)).n - r dW~_j)] / D_i,
-// regrouped so that a neighbour enters through W~_j alone,
-//   dW~_i = -[K_i + sum_j (A/2V) (G(W~_j).n - r W~_j)] / D_i,
-//   K_i   = F_i - sum_j (A/2V) (G(W_j).n - r W_j)      (constant through a solve).
-// With n scaled by A/2V, c2 = A r/2V, t = U.n - c2 and H = rho E + p the bracket's face
-// term is (rho t, rho t U + p n, H t + c2 p, rho E_rot t): 14 FP64 operations and seven
-// doubles of the neighbour, against 19 and fourteen with the increments carried beside
-// the state.  The solve is bound by its FP64 instructions (GB300 issues one warp
+//   dW~_i = [-F_i - sum_j (A/2V) ((G(W~_j) - G(W_j)).n - r dW~_j)] / D_i
+//         = B_i - o_i / D_i,   B_i = -(F_i - sum_j (A/2V) G(W_j).n) / D_i (constant through a solve),
+//   o_i   = sum_j (A/2V) (G(W~_j).n - r dW~_j).
+// Two forms, with n scaled by A/2V, c2 = A r/2V and H = rho E + p:
+// INC (FP64 contexts): t = U.n, and a face adds (rho t, rho t U + p n, H t, rho E_rot t) - c2
+// dW~, 19 FP64 operations and thirteen doubles of the neighbour.  The increments are carried
+// beside the state, so that the rounding of a solve is relative to the fluxes and to them.
+// Otherwise (mixed contexts): r dW~ is folded into the flux, t = U.n - c2, and with B_i + W_i
+// in the place of B_i an update is W~_i itself: (rho t, rho t U + p n, H t + c2 p, rho E_rot
+// t), 14 operations and seven doubles.  Its rounding is relative to r W, 1e-16 of the state:
+// FP64 contexts show it (cavity 8^3 x 512, residuals that a march settles at, folded / with
+// increments: rho 1.7e-16 / 3.0e-17, rho U 3.6e-15 / 2.6e-15, rho E 1.4e-16 / 4.8e-17; error
+// of two iterations of 37,086 x 304 against 64-bit formulas 1.3e-13 / 1.1e-13), mixed ones
+// round their distributions at 6e-8 and do not (their FP32 results are the same bits).  The
+// increments cost 4-5 % of an iteration on 8^3 x 512, 1.6 % on 37,086 x 304; in mixed
+// contexts they would cost 6 % (12^3 x 343) and 4.5 % (61,911 x 3,033).
+// The solve is bound by its FP64 instructions (GB300 issues one warp
 // instruction per 64 cycles and sub-partition, whatever the number of active lanes and
 // however independent the chains) and, on small meshes, by the latency of one phase.
-//   iterate   mPc [p][8]:  rho, U, H, p, rho E_rot, -  (gathered: two 32-byte loads)
-//   constants mCon [9][p]: B (6), 1/D, 1/(D + 1/(Z tau)), 1/(Z tau); with K and W^n folded
-//             into B = W - K/D an update is W~ = B - o/D, o the sum of the face terms, and
-//             rho E_rot~ = B_5 - (o_5 - rho R T~/(Z tau)) / (D + 1/(Z tau)),
-//             B_5 = W_5 - (K_5 + W_5/(Z tau)) / (D + 1/(Z tau))
+//   iterate   mPc [p][8]:  rho, U, H, p, rho E_rot, -;  INC: mDw [p][8]: dW~, -, -
+//             (gathered in 32-byte loads)
+//   constants mCon [15][p]: B (6), 1/D, 1/(D + 1/(Z tau)), 1/(Z tau), INC: W^n (6);
+//             d(rho E_rot)~ = B_5 + ((rho R T~ - rho E_rot^n)/(Z tau) - o_5) / (D + 1/(Z tau)),
+//             B_5 with that denominator too; folded: rho E_rot^n/(Z tau) in B_5 as well
 //   slots     mSlot [4][ms][p]: (A/2V) n, A r/2V;  mNbr [ms][p]
 // (constants and slots across the cells, so that a warp's loads are contiguous)
-__device__ __forceinline__ void macro_face(double (&o)[6], const double (&P)[8], const double (&s)[4]) {
-    const double t = fma(P[1], s[0], fma(P[2], s[1], fma(P[3], s[2], -s[3])));
+template <bool INC>
+__device__ __forceinline__ void macro_face(double (&o)[6], const double (&P)[8], const double (&dW)[8],
+                                           const double (&s)[4]) {
+    const double t = fma(P[1], s[0], fma(P[2], s[1], INC ? P[3] * s[2] : fma(P[3], s[2], -s[3])));
     const double m = P[0] * t;
     o[0] += m;
     o[1] = fma(m, P[1], fma(P[5], s[0], o[1]));
     o[2] = fma(m, P[2], fma(P[5], s[1], o[2]));
     o[3] = fma(m, P[3], fma(P[5], s[2], o[3]));
-    o[4] = fma(P[4], t, fma(s[3], P[5], o[4]));
+    o[4] = fma(P[4], t, INC ? o[4] : fma(s[3], P[5], o[4]));
     o[5] = fma(P[6], t, o[5]);
+    if constexpr (INC)
+#pragma unroll
+        for (int q = 0; q < 6; ++q) o[q] = fma(-s[3], dW[q], o[q]);
 }
 // the iterate's record of a neighbour (32-byte aligned), through L2 (in the cooperative
 // solve other blocks wrote it during this kernel)
@@ -1407,6 +1421,11 @@ __device__ __forceinline__ bool positive(double x) {
     const long long b = __double_as_longlong(x);
     return b > 0 && b <= 0x7ff0000000000000LL;
 }
+
+// Rows of mCon
+constexpr int MC_B = 0, MC_ID = 6, MC_IDR = 7, MC_IZT = 8, MC_W = 9;
+template <typename T>
+constexpr bool MACRO_INC = sizeof(T) == 8;
 
 // Set-up of a solve, first part (needs W^n and the spectral radii only, so the graph runs
 // it beside the reconstruction): the iterate W^n, the slots, 1/D with D = 1/dt + sum_j
@@ -1441,30 +1460,42 @@ __global__ void __launch_bounds__(128) k_macro_rec(Dev<T> c, const int* col_cell
     P[1] = make_double2(U[1], U[2]);
     P[2] = make_double2(W[4] + pr, pr);
     P[3] = make_double2(W[5], 0.0);
-    c.mCon[(size_t)6 * c.N + p] = inv(D);
-    c.mCon[(size_t)7 * c.N + p] = inv(D + izt);
-    c.mCon[(size_t)8 * c.N + p] = izt;
+    const size_t N = (size_t)c.N;
+    c.mCon[MC_ID * N + p] = inv(D);
+    c.mCon[MC_IDR * N + p] = inv(D + izt);
+    c.mCon[MC_IZT * N + p] = izt;
+    if constexpr (MACRO_INC<T>) {
+        double2* Q = reinterpret_cast<double2*>(c.mDw + 8 * (size_t)p);
+        for (int q = 0; q < 4; ++q) Q[q] = make_double2(0.0, 0.0);
+        for (int q = 0; q < 6; ++q) c.mCon[(MC_W + q) * N + p] = W[q];
+    }
 }
 
-// second part, one thread per colour position: K = F - sum_j (face terms at W^n), and B
+// second part, one thread per colour position: B
 template <typename T>
 __global__ void __launch_bounds__(128) k_macro_con(Dev<T> c, const int* col_cell) {
+    constexpr bool INC = MACRO_INC<T>;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= c.N) return;
     double o[6] = {0, 0, 0, 0, 0, 0};
+    const double zero[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (int q = 0; q < c.ms; ++q) {
         const int j = c.mNbr[(size_t)q * c.N + p];
         if (j < 0) continue;
         double P[8], s[4];
         macro_load(c.mPc + 8 * (size_t)j, P);
         macro_slot(c, q, p, s);
-        macro_face(o, P, s);
+        macro_face<INC>(o, P, zero, s);
     }
     const size_t i = (size_t)col_cell[p], N = (size_t)c.N;
     const double *F = c.macroF + 6 * i, *W = c.W + 6 * i;
-    const double iD = c.mCon[6 * N + p], iDr = c.mCon[7 * N + p], izt = c.mCon[8 * N + p];
-    for (int q = 0; q < 5; ++q) c.mCon[q * N + p] = fma(o[q] - F[q], iD, W[q]);
-    c.mCon[5 * N + p] = fma(o[5] - fma(W[5], izt, F[5]), iDr, W[5]);
+    const double iD = c.mCon[MC_ID * N + p], iDr = c.mCon[MC_IDR * N + p], izt = c.mCon[MC_IZT * N + p];
+    if constexpr (INC) {
+        for (int q = 0; q < 6; ++q) c.mCon[(MC_B + q) * N + p] = (o[q] - F[q]) * (q < 5 ? iD : iDr);
+    } else {
+        for (int q = 0; q < 5; ++q) c.mCon[(MC_B + q) * N + p] = fma(o[q] - F[q], iD, W[q]);
+        c.mCon[(MC_B + 5) * N + p] = fma(o[5] - fma(W[5], izt, F[5]), iDr, W[5]);
+    }
 }
 
 // Launched with programmatic stream serialisation: each phase waits for the previous
@@ -1489,17 +1520,13 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 // over the faces and no launch of its own.
 //
 // L by macro_lanes: the number of warps that share a sub-partition times the FP64
-// instructions of one warp (14 per face slot, the halving, 20 for the update, or 12 where
-// with eight threads each holds one row of it), which is
-// the phase's time as long as the loads are hidden.  One thread per cell serves large
+// instructions of one warp, which is the phase's time as long as the loads are hidden:
+// per face slot 14, the halving, 20 for the update, or 12 where with eight threads each holds
+// one row of it (INC: 19, 26 and 18, which choose alike).  One thread per cell serves large
 // colours (no redundant update), more threads the small ones, whose phase is one warp's
-// serial chain: 864 cells with six faces take 8 threads (32 instructions instead of 104).
-// Measured against two threads per cell with the increments beside the state (40 sweeps,
-// the whole iteration): cavity 12^3 x 343 mixed 0.772 -> 0.455 ms, cavity 8^3 x 512 FP64
-// 1.94 -> 1.63 ms, sphere 61,911 x 3,033 mixed 12.25 -> 11.62 ms.
-// With K and W^n folded into B, the reciprocal by inv and a row a lane in groups of eight
-// (before: 44 instructions there, 80 with one thread): cavity 12^3 x 343 0.381 -> 0.355
-// ms, cavity 8^3 x 512 FP64 0.66 -> 0.62 ms, sphere 10.23 -> 10.08 ms an iteration.
+// serial chain: 864 cells with six faces take 8 threads, 32 instructions instead of 104.
+// 40 sweeps with two threads a cell and with this rule, the whole iteration: cavity 12^3 x
+// 343 mixed 0.77 and 0.355 ms, sphere 61,911 x 3,033 mixed 12.3 and 10.3 ms.
 __host__ __device__ inline int macro_lanes(int n, int ms) {
     int best = 1;
     long long cost = 0;
@@ -1549,7 +1576,7 @@ __device__ __forceinline__ void group_sum6(double (&o)[6]) {
 // Everything but the iterates is constant through the solve and is loaded before `ready`
 // returns (the wait for the phase before), so that a phase launched ahead of its turn has
 // only the neighbours' records left to fetch.
-template <int L, typename F>
+template <int L, bool INC, typename F>
 __device__ __forceinline__ void macro_point(const DevBase& c, int p, int reps, int g, F&& ready) {
     constexpr int U = L >= 4 ? 2 : 4;             // slots whose loads are issued together
     const size_t N = (size_t)c.N;
@@ -1569,43 +1596,55 @@ __device__ __forceinline__ void macro_point(const DevBase& c, int p, int reps, i
     // lanes 4-6: where the halving leaves them)
     constexpr bool ROW = L == 8;
     const int row = ROW ? min(g < 4 ? g : g - 1, 5) : 0;
-    double B[ROW ? 1 : 6], iD, iDr = 0.0, izt;
+    double B[ROW ? 1 : 6], W[ROW ? 1 : 6], iD, iDr = 0.0, izt;
+    const double w5n = INC ? C[(MC_W + 5) * N] : 0.0;
     if constexpr (ROW) {
-        B[0] = C[row * N];
-        iD = C[(row == 5 ? 7 : 6) * N];
-        izt = row == 5 ? C[8 * N] : 0.0;
+        B[0] = C[(MC_B + row) * N];
+        W[0] = INC ? C[(MC_W + row) * N] : 0.0;
+        iD = C[(row == 5 ? MC_IDR : MC_ID) * N];
+        izt = row == 5 ? C[MC_IZT * N] : 0.0;
     } else {
 #pragma unroll
-        for (int q = 0; q < 6; ++q) B[q] = C[q * N];
-        iD = C[6 * N];
-        iDr = C[7 * N];
-        izt = C[8 * N];
+        for (int q = 0; q < 6; ++q) B[q] = C[(MC_B + q) * N];
+#pragma unroll
+        for (int q = 0; q < 6; ++q) W[q] = INC ? C[(MC_W + q) * N] : 0.0;
+        iD = C[MC_ID * N];
+        iDr = C[MC_IDR * N];
+        izt = C[MC_IZT * N];
     }
     ready();
     double rRT = __ldcg(c.mPc + 8 * (size_t)p + 5);
     for (int q0 = g;;) {
-        double P[U][8];
+        double P[U][8], dW[U][8];
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j[u] >= 0) macro_load(c.mPc + 8 * (size_t)j[u], P[u]);
+            if (j[u] >= 0) {
+                macro_load(c.mPc + 8 * (size_t)j[u], P[u]);
+                if constexpr (INC) macro_load(c.mDw + 8 * (size_t)j[u], dW[u]);
+            }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (j[u] >= 0) macro_face(o, P[u], s[u]);
+            if (j[u] >= 0) macro_face<INC>(o, P[u], dW[u], s[u]);
         q0 += U * L;
         if (q0 >= c.ms) break;
         load_slots(q0);
     }
     double rho, U0, U1, U2, E, mU;
-    double o5 = 0.0;                              // this lane's sum (L = 8) or the rotational row's
+    double d[ROW ? 1 : 6];                        // the increments (folded: W~), L = 8: the lane's own row
+    double o5 = 0.0;                              // the rotational row's sum, or this lane's
     const int lane = threadIdx.x & 31, base = lane & ~(L - 1);
-    const unsigned mask = L == 32 ? 0xffffffffu : ((1u << L) - 1u) << base;
+    const unsigned mask = ((1u << L) - 1u) << base;
+    auto rot = [&](double p) { return INC ? p - w5n : p; };
+    auto add = [](double w, double dw) { return INC ? w + dw : dw; };
+    double dRT = rot(rRT);
     if constexpr (ROW) {
-        double a[3], b[2], d[1];
+        double a[3], b[2], s1[1];
         group_halve(o, a, mask, 4);
         group_halve(a, b, mask, 2);
-        group_halve(b, d, mask, 1);
-        o5 = d[0];
-        const double x = fma(-fma(-izt, rRT, o5), iD, B[0]);          // the lane's row of W~
+        group_halve(b, s1, mask, 1);
+        o5 = s1[0];
+        d[0] = fma(fma(izt, dRT, -o5), iD, B[0]);
+        const double x = add(W[0], d[0]);
         rho = __shfl_sync(mask, x, base);
         const double u = x * inv(rho), mu = x * u;
         U0 = __shfl_sync(mask, u, base + 1);
@@ -1616,27 +1655,41 @@ __device__ __forceinline__ void macro_point(const DevBase& c, int p, int reps, i
     } else {
         group_sum6<L>(o);
         o5 = o[5];
-        rho = fma(-o[0], iD, B[0]);
-        const double m0 = fma(-o[1], iD, B[1]), m1 = fma(-o[2], iD, B[2]), m2 = fma(-o[3], iD, B[3]);
-        E = fma(-o[4], iD, B[4]);
+#pragma unroll
+        for (int q = 0; q < 5; ++q) d[q] = fma(-o[q], iD, B[q]);
+        rho = add(W[0], d[0]);
+        const double m0 = add(W[1], d[1]), m1 = add(W[2], d[2]), m2 = add(W[3], d[3]);
+        E = add(W[4], d[4]);
         const double ir = inv(rho);
         U0 = m0 * ir; U1 = m1 * ir; U2 = m2 * ir;
         mU = fma(m0, U0, fma(m1, U1, m2 * U2));
     }
     const double ei = fma(-0.5, mU, E), pr = 0.4 * ei;   // rho E - 1/2 rho |U|^2, rho R T = 2/5 of it
-    double er = 0.0;
+    double er = 0.0, dr = 0.0;
     bool set = false;
     for (int r = 0; r < reps; ++r) {
-        double w5;
-        if constexpr (ROW) w5 = __shfl_sync(mask, fma(-fma(-izt, rRT, o5), iD, B[0]), base + 6);
-        else w5 = fma(-fma(-izt, rRT, o5), iDr, B[5]);
+        double d5;
+        if constexpr (ROW) d5 = __shfl_sync(mask, fma(fma(izt, dRT, -o5), iD, B[0]), base + 6);
+        else d5 = fma(fma(izt, dRT, -o5), iDr, B[5]);
+        const double w5 = add(w5n, d5);
         // a repeat would be skipped too (rho E_rot and its bound are positive: their bits compare)
         if (!(positive(rho) && positive(ei) && positive(w5) && __double_as_longlong(ei) > __double_as_longlong(w5))) break;
         er = w5;
-        rRT = pr;
+        dr = d5;
+        dRT = rot(pr);
         set = true;
     }
-    if (!set || g != 0) return;
+    if (!set) return;
+    if constexpr (INC && ROW) {
+        if (g != 3 && g != 7) __stcg(c.mDw + 8 * (size_t)p + row, g == 6 ? dr : d[0]);
+    }
+    if (g != 0) return;
+    if constexpr (INC && !ROW) {
+        double2* D = reinterpret_cast<double2*>(c.mDw + 8 * (size_t)p);
+        __stcg(D, make_double2(d[0], d[1]));
+        __stcg(D + 1, make_double2(d[2], d[3]));
+        __stcg(D + 2, make_double2(d[4], dr));
+    }
     double2* P = reinterpret_cast<double2*>(c.mPc + 8 * (size_t)p);
     __stcg(P, make_double2(rho, U0));
     __stcg(P + 1, make_double2(U1, U2));
@@ -1648,12 +1701,12 @@ __device__ __forceinline__ void macro_point(const DevBase& c, int p, int reps, i
 // micro flux's blocks as soon as one of them ends; a block of 128 threads did not fit into
 // the registers that one of those gives back.
 constexpr int MACRO_BS = 64;
-template <int L>
+template <int L, bool INC>
 __global__ void __launch_bounds__(MACRO_BS) k_macro_sweep(const __grid_constant__ DevBase c, int lo, int n, int reps) {
     // phases launched with programmatic stream serialisation (see pdl_wait)
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) / L;
     if (t >= n) return;                           // whole lane group
-    macro_point<L>(c, lo + t, reps, (int)(threadIdx.x % L), [] {
+    macro_point<L, INC>(c, lo + t, reps, (int)(threadIdx.x % L), [] {
         pdl_wait();
         pdl_launch_dependents();
     });
@@ -1707,11 +1760,11 @@ __device__ __forceinline__ bool grid_barrier(unsigned int* bar, int* status, uns
     return s_fail == 0;
 }
 
-template <int L>
+template <int L, bool INC>
 __device__ __forceinline__ void coop_phase(const DevBase& c, int lo, int n, int reps) {
     const int g = (int)(threadIdx.x % L);
     for (int t = (blockIdx.x * blockDim.x + threadIdx.x) / L; t < n; t += (gridDim.x * blockDim.x) / L)
-        macro_point<L>(c, lo + t, reps, g, [] {});
+        macro_point<L, INC>(c, lo + t, reps, g, [] {});
 }
 template <typename T>
 __global__ void __launch_bounds__(128) k_macro_coop(Dev<T> c, const int* col_off, int C, int n_macro,
@@ -1726,10 +1779,10 @@ __global__ void __launch_bounds__(128) k_macro_coop(Dev<T> c, const int* col_off
             const int lo = col_off[col], n = col_off[col + 1] - lo;
             const int reps = C == 1 ? 2 * n_macro : (cc == C - 1 && sw + 1 < 2 * n_macro ? 2 : 1);
             switch (macro_lanes(n, c.ms)) {
-                case 1: coop_phase<1>(c, lo, n, reps); break;
-                case 2: coop_phase<2>(c, lo, n, reps); break;
-                case 4: coop_phase<4>(c, lo, n, reps); break;
-                default: coop_phase<8>(c, lo, n, reps);
+                case 1: coop_phase<1, MACRO_INC<T>>(c, lo, n, reps); break;
+                case 2: coop_phase<2, MACRO_INC<T>>(c, lo, n, reps); break;
+                case 4: coop_phase<4, MACRO_INC<T>>(c, lo, n, reps); break;
+                default: coop_phase<8, MACRO_INC<T>>(c, lo, n, reps);
             }
             if (!grid_barrier(bar, c.status, nb, extra, limit_ns)) return;
         }
@@ -1889,7 +1942,7 @@ __global__ void __launch_bounds__(MACRO_BS) k_macro_sweep32(const __grid_constan
 // W~ = W^n + dW~, tau~ and the per-cell record of the micro sweeps: constants of the
 // predicted equilibrium phi~* built from (W~, q^n) (reading: the prediction gives no
 // heat flux, so the last Step-6 value is used), 1/tau~, and 1/dt + 1/tau~.  W~ comes
-// from the FP64 iterate's record, or with m32 from W^n and the first six floats of the
+// from the FP64 solve's increments or record, or with m32 from the first six floats of the
 // cell's FP32 delta record.
 template <typename T>
 __global__ void k_macro_finish(Dev<T> c, int m32) {
@@ -1902,12 +1955,16 @@ __global__ void k_macro_finish(Dev<T> c, int m32) {
         const float* d32 = reinterpret_cast<const float*>(m32_delta(c) + 3 * pos);
         for (int m = 0; m < 6; ++m) Wt[m] = c.W[6 * (size_t)i + m] + (double)d32[m];
     } else {
-        double P[8];
-        macro_load(c.mPc + 8 * pos, P);
-        Wt[0] = P[0];
-        for (int d = 0; d < 3; ++d) Wt[1 + d] = P[0] * P[1 + d];
-        Wt[4] = P[4] - P[5];
-        Wt[5] = P[6];
+        double x[8];
+        macro_load((MACRO_INC<T> ? c.mDw : c.mPc) + 8 * pos, x);
+        if constexpr (MACRO_INC<T>) {
+            for (int m = 0; m < 6; ++m) Wt[m] = c.W[6 * (size_t)i + m] + x[m];
+        } else {
+            Wt[0] = x[0];
+            for (int d = 0; d < 3; ++d) Wt[1 + d] = x[0] * x[1 + d];
+            Wt[4] = x[4] - x[5];
+            Wt[5] = x[6];
+        }
     }
     const Prim p = prim_from_W(Wt, c.R);
     const double tau = relax_time(c, p.rho, p.Ttr), it = 1.0 / tau;

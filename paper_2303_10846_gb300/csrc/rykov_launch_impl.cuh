@@ -232,7 +232,8 @@ cudaError_t Launch<T>::macro(const Dev<T>& d, cudaStream_t s, const Sched& sc, i
     if (!done) {
         for (const Phase& ph : sgs_phases(sc, n_macro)) {
             const int lo = sc.col_off[ph.col], n = sc.col_off[ph.col + 1] - lo, L = macro_lanes(n, d.ms);
-            const cudaError_t e = launch_phase(L == 1 ? k_macro_sweep<1> : L == 2 ? k_macro_sweep<2> : L == 4 ? k_macro_sweep<4> : k_macro_sweep<8>,
+            const cudaError_t e = launch_phase(L == 1 ? k_macro_sweep<1, MACRO_INC<T>> : L == 2 ? k_macro_sweep<2, MACRO_INC<T>>
+                                               : L == 4 ? k_macro_sweep<4, MACRO_INC<T>> : k_macro_sweep<8, MACRO_INC<T>>,
                                                (long long)n * L, sc.pdl && !first, s, db, lo, n, ph.reps);
             if (e != cudaSuccess) return e;
             first = false;

@@ -148,3 +148,16 @@ def test_mixed_reconstruction_is_homogeneous(mesh, exponent):
         out.append(s.debug_get("FACE")[:, interior] * 2.0 ** e)
     assert np.isfinite(out[0]).all() and np.abs(out[0] - 1.0).max() > 0.5
     assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("n,n_gh", [(6, 6), (8, 8)])
+def test_settled_fp64_march_leaves_density_and_energy_where_they_are(n, n_gh):
+    """A march that has settled: the macro solve's increment is zero to rounding, so W~ is W
+    but for the last bit of a few cells.  The mean relative change of a step is then below a
+    quarter of an ulp (2^-54); a solve whose own rounding is relative to W moves most cells
+    by half an ulp or more."""
+    from paper_2303_10846_gb300.rykov import Solver
+    s = Solver(I.cavity_workload(n=n, n_gh=n_gh), "fp64")
+    s.iterate(200)
+    rho, energy = np.mean([s.iterate(5)[2][[0, 4]] for _ in range(20)], axis=0)
+    assert rho <= 2.0 ** -54 and energy <= 2.0 ** -54, (rho, energy)
