@@ -28,7 +28,7 @@ constexpr int ADJ_FPAR = 12;     // per boundary face: dR/dp^T v (6), J, force (
 // records of the state (written once per state): equilibrium constants of a cell or an
 // interior face (EQA), the face's moments (FMOM, as the forward kernels'), and the sums
 // over the velocities that depend on v
-constexpr int EQA = 28, ADJ_NS = 15, ADJ_CS = 20, ADJ_FS = 17, ADJ_FC = 16;
+constexpr int EQA = 22, ADJ_NS = 15, ADJ_CS = 20, ADJ_FS = 17, ADJ_FC = 16;
 
 // Arrays in the arithmetic type S of the per-velocity work: FP64, or FP32 for mixed
 // contexts, whose vectors, scalars and sums stay FP64
@@ -115,20 +115,22 @@ static_assert(sizeof(Acc<double>) == sizeof(double), "running FP64 sums are an a
 // For weights (Gb, Hb) of (G*, R*) the derivatives with respect to the state are sums over
 // the velocities of a few products, with P = (Gb + theta_rot Hb) M_t, Q = Hb M_t,
 // P' = (Gb + theta Hb) M, Q' = Hb M, E = P (1 + s A_t) + B_t r Q, E' likewise,
-// v1 = B_t Q + B Q', v2 = P A_t + P' A, a = 1/(15 rho theta_tr^3), a' = w0/(15 rho theta^3):
+// v1 = B_t Q + B Q', v2 = P A_t + P' A, y = |c|^2/theta, k' = w0/(15 rho theta^2), y_t and k alike:
 //   rho          (1/rho) sum (P + P')          (the heat-flux terms cancel)
 //   theta_rot    sum Q (1 + s A_t)
-//   theta        sum Q' (1 + s A) - (B/theta) r Q' + a' s P' (10 - 3 |c|^2/theta)
-//                    + E' (|c|^2/(2 theta^2) - 3/(2 theta));   theta_tr likewise without the first
+//   theta        (1/theta) sum theta Q' (1 + s A) - B r Q' + k' s P' (10 - 3 y) + E' (y - 3)/2;
+//                theta_tr likewise without the first
 //   q_rot, q_tr  sum v1 c, sum v2 c
-//   U            sum (E/theta_tr + E'/theta - 2 a s P - 2 a' s P') c - q_rot sum v1 - q_tr sum v2
+//   U            sum ((E - 2 k s P)/theta_tr + (E' - 2 k' s P')/theta) c - q_rot sum v1 - q_tr sum v2
 // Fifteen sums and about 95 operations a velocity, against 190 for the chain rule written
-// out term by term.  Sums: 0 rho, 1 theta_rot, 2 theta, 3 theta_tr, 4 v1, 5 v2,
-// 6-8 v1 c, 9-11 v2 c, 12-14 the U sum.
+// out term by term.  Sums: 0 rho, 1 theta_rot, 2 theta, 3 theta_tr (2 and 3 without the
+// factors 1/theta), 4 v1, 5 v2, 6-8 v1 c, 9-11 v2 c, 12-14 the U sum.  No constant has more
+// than 1/(rho theta^2) in it, so that FP32 serves any units that the forward form does
+// (with 1/(rho theta^4), theta = 7e10 lost the derivatives of the temperatures).
 // Constants (EqA, EQA values in memory): see eqa_make.
 template <typename S>
 struct EqA {
-    S U[3], qt[3], qr[3], thr, th, nt, n, xt, x, ka, kb, kc, kd, Bt, B, itr, it, zt0, zt1, z0, z1, ib;
+    S U[3], qt[3], qr[3], thr, th, nt, n, ka, kb, kc, kd, Bt, B, itr, it, ib;
 };
 static_assert(sizeof(EqA<double>) == EQA * sizeof(double), "EQA");
 // scale: factor on the Maxwellians (the blend's weight b at a face; ib = 1/b)
@@ -136,7 +138,7 @@ template <typename S, typename T>
 __device__ __forceinline__ EqA<S> eqa_make(const Dev<T>& c, double rho, const double* U, double T_, double Ttr,
                                            double Trot, const double* qtr, const double* qrot, double scale) {
     const double th = c.R * T_, tt = c.R * Ttr, it = 1.0 / th, itr = 1.0 / tt, ir = 1.0 / rho;
-    const double i15 = ir / 15.0, l2e = 1.4426950408889634;
+    const double i15 = ir / 15.0;
     EqA<S> e;
     for (int k = 0; k < 3; ++k) { e.U[k] = (S)U[k]; e.qt[k] = (S)qtr[k]; e.qr[k] = (S)qrot[k]; }
     e.thr = (S)(c.R * Trot);
@@ -144,16 +146,12 @@ __device__ __forceinline__ EqA<S> eqa_make(const Dev<T>& c, double rho, const do
     const double at = 2.0 * PI * tt, ar = 2.0 * PI * th;
     e.nt = (S)(scale * (1.0 - 1.0 / c.Z) * rho / (at * sqrt(at)));
     e.n = (S)(scale / c.Z * rho / (ar * sqrt(ar)));
-    e.xt = (S)(-0.5 * l2e * itr);
-    e.x = (S)(-0.5 * l2e * it);
-    const double ka = itr * itr * itr * i15, kc = c.omega0 * it * it * it * i15;
-    e.ka = (S)ka; e.kb = (S)(-5.0 * ka * tt);
-    e.kc = (S)kc; e.kd = (S)(-5.0 * kc * th);
+    const double ka = itr * itr * i15, kc = c.omega0 * it * it * i15;
+    e.ka = (S)ka; e.kb = (S)(-5.0 * ka);
+    e.kc = (S)kc; e.kd = (S)(-5.0 * kc);
     e.Bt = (S)((1.0 - c.delta) * ir * itr);
     e.B = (S)(c.omega1 * (1.0 - c.delta) * ir * it);
     e.itr = (S)itr; e.it = (S)it;
-    e.zt0 = (S)(10.0 * ka); e.zt1 = (S)(-3.0 * ka * itr);
-    e.z0 = (S)(10.0 * kc); e.z1 = (S)(-3.0 * kc * it);
     e.ib = (S)(1.0 / scale);
     return e;
 }
@@ -164,49 +162,47 @@ __device__ __forceinline__ void eqa_terms(const EqA<S>& e, S ux, S uy, S uz, S G
     const S c2 = cx * cx + cy * cy + cz * cz;
     const S s = cx * e.qt[0] + cy * e.qt[1] + cz * e.qt[2];
     const S r = cx * e.qr[0] + cy * e.qr[1] + cz * e.qr[2];
-    const S Mt = e.nt * ex2(c2 * e.xt), M = e.n * ex2(c2 * e.x);
-    const S At = c2 * e.ka + e.kb, A = c2 * e.kc + e.kd;
+    const S yt = c2 * e.itr, y = c2 * e.it, hl = S(-0.5 * 1.4426950408889634);
+    const S Mt = e.nt * ex2(yt * hl), M = e.n * ex2(y * hl);
+    const S At = yt * e.ka + e.kb, A = y * e.kc + e.kd;
     const S sAt = s * At, sA = s * A;
     const S Gt = Mt * sAt + Mt, Gr = M * sA + M;
     const S BM = e.Bt * Mt + e.B * M;
     G = Gt + Gr;
     H = e.thr * Gt + (e.th * Gr + r * BM);
     const S P = (Hb * e.thr + Gb) * Mt, Q = Hb * Mt, P1 = (Hb * e.th + Gb) * M, Q1 = Hb * M;
-    const S Qr = Q * r * e.Bt, Q1r = Q1 * r * e.B, Ps = P * s, P1s = P1 * s;
-    const S E = P * sAt + (P + Qr), E1 = P1 * sA + (P1 + Q1r);
+    const S Qr = Q * r * e.Bt, Q1r = Q1 * r * e.B, kP = P * s * e.ka, kP1 = P1 * s * e.kc;
+    const S E = P * sAt + (P + Qr), E1 = P1 * sA + (P1 + Q1r), tQ = e.th * Q1;
     t[0] += P + P1;
     t[1] += Q * sAt + Q;
-    // |c|^2/(2 theta^2) - 3/(2 theta) = (|c|^2/theta - 3) / (2 theta)
-    const S hw = S(0.5) * e.it, hwt = S(0.5) * e.itr;
-    const S w1 = (c2 * e.it - S(3)) * hw, w1t = (c2 * e.itr - S(3)) * hwt;
-    t[2] += Q1 * sA + Q1;
-    t[2] += P1s * (c2 * e.z1 + e.z0);
-    t[2] += E1 * w1;
-    t[2] -= Q1r * e.it;
-    t[3] += Ps * (c2 * e.zt1 + e.zt0);
-    t[3] += E * w1t;
-    t[3] -= Qr * e.itr;
+    t[2] += tQ * sA + tQ;
+    t[2] += kP1 * (S(10) - S(3) * y);
+    t[2] += E1 * (S(0.5) * y - S(1.5));
+    t[2] -= Q1r;
+    t[3] += kP * (S(10) - S(3) * yt);
+    t[3] += E * (S(0.5) * yt - S(1.5));
+    t[3] -= Qr;
     const S v1 = Hb * BM, v2 = P * At + P1 * A;
     t[4] += v1;
     t[5] += v2;
     t[6] += v1 * cx; t[7] += v1 * cy; t[8] += v1 * cz;
     t[9] += v2 * cx; t[10] += v2 * cy; t[11] += v2 * cz;
-    const S g = E * e.itr + E1 * e.it - S(2) * (e.ka * Ps + e.kc * P1s);
+    const S g = e.itr * (E - S(2) * kP) + e.it * (E1 - S(2) * kP1);
     t[12] += g * cx; t[13] += g * cy; t[14] += g * cz;
 }
 // derivatives with respect to (rho, U, theta, theta_tr, theta_rot, q_tr, q_rot) from the
 // fifteen sums (d in the order of the comment above eqa_terms' formulas: 0 rho, 1-3 U,
 // 4 theta, 5 theta_tr, 6 theta_rot, 7-9 q_tr, 10-12 q_rot)
-__device__ __forceinline__ void eqa_grad(const double* t, double rho, const double* qtr, const double* qrot,
-                                         double (&d)[13]) {
+__device__ __forceinline__ void eqa_grad(const double* t, double rho, double th, double tt, const double* qtr,
+                                         const double* qrot, double (&d)[13]) {
     d[0] = t[0] / rho;
     for (int k = 0; k < 3; ++k) {
         d[1 + k] = t[12 + k] - qrot[k] * t[4] - qtr[k] * t[5];
         d[7 + k] = t[9 + k];
         d[10 + k] = t[6 + k];
     }
-    d[4] = t[2];
-    d[5] = t[3];
+    d[4] = t[2] / th;
+    d[5] = t[3] / tt;
     d[6] = t[1];
 }
 
@@ -316,7 +312,7 @@ __global__ void __launch_bounds__(64) k_adj_crev(Dev<double> c, AdjBufs a) {
     adj_sums<S>(a.csum + (size_t)i * ADJ_CS, t);
     const double *vW = a.vW + 6 * (size_t)i, *vq = a.vq + 6 * (size_t)i;
     double d[13];
-    eqa_grad(t, p.rho, q, q + 3, d);
+    eqa_grad(t, p.rho, R * p.T, R * p.Ttr, q, q + 3, d);
     double rb = d[0], Ub[3];
     for (int k = 0; k < 3; ++k) Ub[k] = d[1 + k] - 0.5 * vq[k] * t[16] - t[17 + k];
     double Tb = R * d[4], Ttrb = R * d[5], Trotb = R * d[6];
@@ -607,7 +603,7 @@ __global__ void __launch_bounds__(64) k_adj_frev(Dev<double> c, AdjBufs a, AdjAr
     adj_sums<S>(a.fsum + (size_t)fi * (ADJ_FS + 1), t);
     const double rho = f.rho, tau = f.tau, ts = tau + s;
     double d[13];
-    eqa_grad(t, rho, f.qtr, f.qrot, d);
+    eqa_grad(t, rho, Rg * f.T, Rg * f.Ttr, f.qtr, f.qrot, d);
     double rb = d[0], Ub[3] = {d[1], d[2], d[3]};
     double Tb = Rg * d[4], Ttrb = Rg * d[5], Trotb = Rg * d[6], taub = t[15] * s / (ts * ts);
     double Qtb[3], Qrb[3];

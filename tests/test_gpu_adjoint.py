@@ -385,3 +385,37 @@ def test_mixed_boundary_terms_are_fp64_and_rounded_once(monkeypatch):
     a, b = (x[:2 * s.N * s.K].reshape(2, s.N, s.K)[:, one] for x in (g, g64))
     assert one.sum() > 10 and np.abs(b).max() > 0
     assert (np.abs(a - b) <= 2.0 ** -24 * (1 + 1e-6) * np.abs(b)).all()
+
+
+@pytest.mark.parametrize("prec,b", [("mixed", 18), ("mixed", -12), ("fp64", 18)])
+def test_adjoint_product_in_other_units_of_velocity(prec, b):
+    """Velocities times c = 2^b (the gas constant, the viscosity and the weights with them;
+    18: metres to some hundredths of a millimetre per second): the products of the two unit
+    systems agree to the tolerances of the precisions.  X scales as (c^-3 | 1, c, c, c, c^2,
+    c^2 | c^3), R as (c^-2 | as X | as X), the product of v/R as 1/X; first order (the FP32
+    limiter derivative has an absolute threshold)."""
+    import copy
+    base = TW.tiny_tet(n_gh=5, lim=2, cfl_imp=20.0)
+    wl = copy.deepcopy(base)
+    c = 2.0 ** b
+    wl.prim0[:, 1:4] *= c
+    wl.dvs = I.DVS(u=base.dvs.u * c, w=base.dvs.w * c ** 3)
+    wl.params.R *= c * c
+    wl.params.mu_ref *= c
+    wl.bcs = [I.BC(q.kind, q.rho, tuple(x * c for x in q.U), q.T) for q in base.bcs]
+    s = _solver_prec(base, prec, 2)
+    s.iterate(3)
+    N, K = s.N, s.K
+    tail = np.concatenate([np.tile([1.0, c, c, c, c * c, c * c], N), np.full(6 * N, c ** 3)])
+    X = np.concatenate([np.full(2 * N * K, c ** -3), tail])
+    X[N * K:2 * N * K] = c ** -1
+    R = np.concatenate([np.full(2 * N * K, c ** -2), tail])
+    R[N * K:2 * N * K] = 1.0
+    v = np.random.default_rng(12).standard_normal(s.state_len)
+    out, _ = s.vjp(v)
+    t = _solver_prec(wl, prec, 2)
+    t.put_state(s.get_state() * X)
+    scaled, _ = t.vjp(v / R)
+    st = Steady(base)
+    for p, q in zip(_blocks(st, scaled * X), _blocks(st, out)):
+        assert _rel(p, q) < (1e-10 if prec == "fp64" else 1e-5)
