@@ -477,12 +477,8 @@ __global__ void __launch_bounds__(WPB * 32) k_adj_mom(Dev<double> c, AdjBufs a, 
     const int f = c.face_int[fi];
     const S* g0 = r.f0 + (size_t)f * c.Kp;
     const S* h0 = g0 + (size_t)c.F * c.Kp;
-    const float wv = lane < 8 ? (float)c.W[6 * (size_t)c.fc[2 * f + (lane >> 2)] + (lane & 3)] : 1.f;
-    const float ia = 1.f / __shfl_sync(0xffffffffu, wv, 0), ib = 1.f / __shfl_sync(0xffffffffu, wv, 4);
     float Ur[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        Ur[d] = 0.5f * (__shfl_sync(0xffffffffu, wv, 1 + d) * ia + __shfl_sync(0xffffffffu, wv, 5 + d) * ib);
+    face_ref_velocity(c, f, lane, Ur);
     AdjSum<S, 17> m;
     for (int k0 = NV * lane; k0 < c.K; k0 += 32 * NV) {
         S ux[NV], uy[NV], uz[NV], w[NV], g[NV], h[NV];

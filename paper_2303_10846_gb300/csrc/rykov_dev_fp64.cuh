@@ -26,14 +26,15 @@ __device__ __forceinline__ void min_bits(unsigned long long& m, double x) {
     m = b > m ? b : m;
 }
 // u.n > 0 as the rounded FP64 dot product (dot_rn) has it.  The FP32 product with rounded
-// u and n is off by less than 4e-7 |u|_1 (|n| <= 1), so beyond thr = 1e-6 |u|_1 its sign
-// is the sign; closer, the FP64 product decides.
+// u and n is off by less than 4e-7 |u|_1 (|n| <= 1) and, among subnormal numbers, 1e-44, so
+// beyond thr = 1e-6 |u|_1 + 1e-43 its sign is the sign; closer, the FP64 product decides
+// (beyond the range of FP32 too: thr is infinite there).
 struct VelF {
     float x, y, z, thr;
 };
 __device__ __forceinline__ VelF vel_f(const DevBase& c, int k) {
     const float x = c.uF[k], y = c.uF[c.Kp + k], z = c.uF[2 * c.Kp + k];
-    return VelF{x, y, z, 1e-6f * (fabsf(x) + fabsf(y) + fabsf(z))};
+    return VelF{x, y, z, fmaf(1e-6f, fabsf(x) + fabsf(y) + fabsf(z), 1e-43f)};
 }
 __device__ __forceinline__ bool outflow(const VelF& u, float4 n, double ux, double uy, double uz, double nx,
                                         double ny, double nz) {
@@ -336,13 +337,9 @@ __global__ void __launch_bounds__(WPB * 32) k_face_mom_d(Dev<double> c) {
     const int f = c.face_int[fi];
     const double* g0 = c.face + (size_t)f * c.Kp;
     const double* h0 = g0 + (size_t)c.F * c.Kp;
-    // reference velocity U_r, the mean of the cells' U^n (any value is exact: in FP32)
-    const float wv = lane < 8 ? (float)c.W[6 * (size_t)c.fc[2 * f + (lane >> 2)] + (lane & 3)] : 1.f;
-    const float ia = 1.f / __shfl_sync(0xffffffffu, wv, 0), ib = 1.f / __shfl_sync(0xffffffffu, wv, 4);
-    double Ur[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        Ur[d] = (double)(0.5f * (__shfl_sync(0xffffffffu, wv, 1 + d) * ia + __shfl_sync(0xffffffffu, wv, 5 + d) * ib));
+    float Uf[3];
+    face_ref_velocity(c, f, lane, Uf);
+    const double Ur[3] = {(double)Uf[0], (double)Uf[1], (double)Uf[2]};
     double m[17];
 #pragma unroll
     for (int j = 0; j < 17; ++j) m[j] = 0.0;

@@ -494,13 +494,8 @@ __global__ void __launch_bounds__(WPB * 32, 2) k_face_interior_p(Dev<float> c) {
         const float4 a = s_r[wib][it % FACE_ST][0][lane], b = s_r[wib][it % FACE_ST][1][lane];
         return RowPair{Row4{{lo2(a), hi2(a)}}, Row4{{lo2(b), hi2(b)}}};
     };
-    // reference velocity U_r: the mean of the cells' U^n (any value is exact)
-    const float wv = lane < 8 ? (float)c.W[6 * (size_t)c.fc[2 * f + (lane >> 2)] + (lane & 3)] : 1.f;
-    const float ia = 1.f / __shfl_sync(0xffffffffu, wv, 0), ib = 1.f / __shfl_sync(0xffffffffu, wv, 4);
     float Ur[3];
-#pragma unroll
-    for (int d = 0; d < 3; ++d)
-        Ur[d] = 0.5f * (__shfl_sync(0xffffffffu, wv, 1 + d) * ia + __shfl_sync(0xffffffffu, wv, 5 + d) * ib);
+    face_ref_velocity(c, f, lane, Ur);
     FF v[17];
     {
         const float2 mx = f2(-Ur[0]), my = f2(-Ur[1]), mz = f2(-Ur[2]);

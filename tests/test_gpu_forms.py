@@ -161,3 +161,42 @@ def test_settled_fp64_march_leaves_density_and_energy_where_they_are(n, n_gh):
     s.iterate(200)
     rho, energy = np.mean([s.iterate(5)[2][[0, 4]] for _ in range(20)], axis=0)
     assert rho <= 2.0 ** -54 and energy <= 2.0 ** -54, (rho, energy)
+
+
+@pytest.mark.parametrize("a,b,product", [(200, 0, True), (0, 140, False), (160, 135, True), (-200, -140, False)])
+def test_fp64_scheme_has_the_range_of_fp64(a, b, product):
+    """Densities times 2^-a and velocities times 2^-b (the gas constant, the viscosity and
+    the weights with them) scale the fields by powers of two: beyond the range of FP32 the
+    march, the wall sums and the steady residual are the unscaled ones to rounding (1e-10,
+    the tolerance of FP64 parity), and the adjoint product is finite (product: where the
+    squared denominators of its limiter, products of four values of the distribution, are)."""
+    import copy
+    from paper_2303_10846_gb300.rykov import Solver
+    from tests import workloads as TW
+    base = TW.tiny_tet(n_gh=5, cfl_imp=20.0)
+    wl = copy.deepcopy(base)
+    r, c = 2.0 ** -a, 2.0 ** -b
+    wl.prim0[:, 0] *= r
+    wl.prim0[:, 1:4] *= c
+    wl.dvs = I.DVS(u=base.dvs.u * c, w=base.dvs.w * c ** 3)
+    wl.params.R *= c * c
+    wl.params.mu_ref *= r * c
+    wl.bcs = [I.BC(q.kind, q.rho * r, tuple(x * c for x in q.U), q.T) for q in base.bcs]
+    wl.ref = dict(rho=r, U=tuple(x * c for x in base.ref["U"]), T=base.ref["T"])
+    out = []
+    for w in (base, wl):
+        s = Solver(w, "fp64")
+        s.bind_adjoint(2)
+        s.iterate(3)
+        W, q, _ = s.moments()
+        per = s.surface()[0]
+        R = s.steady_residual()[:2 * s.N * s.K].reshape(2, -1)
+        v = s.vjp(np.ones(s.state_len))[0]
+        out.append((W, q, per[:, :5], R, v))
+    x, y = out
+    scales = (np.array([r, r * c, r * c, r * c, r * c * c, r * c * c]), r * c ** 3,
+              np.array([r * c * c] * 4 + [r * c ** 3]), np.array([[r / c ** 2], [r]]))
+    for p, q, sc in zip(x, y, scales):
+        z = q / sc
+        assert np.abs(z - p).max() <= 1e-10 * np.abs(p).max()
+    assert not product or np.isfinite(y[4]).all()
