@@ -352,13 +352,10 @@ static int bind_impl(rk_ctx* ctx, rk::Dev<T>& d) {
     for (size_t f = 0; f < F; ++f)
         for (int r = 0; r < 3; ++r) { fns[r * F + f] = ctx->fn[3 * f + r]; fxs[r * F + f] = ctx->fx[3 * f + r]; }
     std::vector<double> us(3 * Kp, 0.0), ws(Kp, 0.0);
-    // The velocities of the K padding of FP32 contexts lie a hundred times beyond the
-    // largest one (weight zero), where every Maxwellian underflows to zero: the kernels
-    // need not mask the equilibria there
-    double umax = 0.0;
-    if (sizeof(T) == 4)
-        for (double x : ctx->u) umax = std::max(umax, std::fabs(x));
-    std::vector<T> uTs(3 * Kp, (T)(100.0 * umax)), wTs(Kp, T(0));
+    // The K padding of FP32 contexts repeats the last velocity with weight zero: the kernels
+    // evaluate the equilibria there without a mask and add them times that zero, so they have
+    // to be finite where those of the real velocities are
+    std::vector<T> uTs(3 * Kp, T(0)), wTs(Kp, T(0));
     std::vector<float> uFs(3 * Kp, 0.f);
     std::vector<double> u2s(Kp, 0.0);
     for (size_t k = 0; k < K; ++k) {
@@ -367,6 +364,9 @@ static int bind_impl(rk_ctx* ctx, rk::Dev<T>& d) {
         ws[k] = ctx->w[k];
         wTs[k] = (T)ctx->w[k];
     }
+    if (sizeof(T) == 4)
+        for (size_t k = K; k < Kp; ++k)
+            for (int r = 0; r < 3; ++r) uTs[r * Kp + k] = uTs[r * Kp + K - 1];
     ctx->wall_b.clear();
     for (int b = 0; b < ctx->Fb; ++b) {
         int bc = -1 - ctx->fc32[2 * (size_t)ctx->face_bnd[b] + 1];

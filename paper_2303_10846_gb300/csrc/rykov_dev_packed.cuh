@@ -434,8 +434,8 @@ __global__ void __launch_bounds__(WPB * 32, RECONP_MINB * 8 / WPB)
 // That leaves room for two blocks of eight warps per SM only, too few to hide the rows'
 // latency, so the rows come FACE_ST - 1 steps ahead as asynchronous copies (with one step
 // in registers instead the kernel was slower than the scalar form: 9.1 ms against 7.9 on
-// 262,000 faces x 5,991).  No select guards the K padding: its velocities lie far outside
-// the velocity space, so phi* vanishes there (see bind_impl).
+// 262,000 faces x 5,991).  No select guards the K padding: it repeats the last velocity with
+// weight zero (see bind_impl), its face values are in no sum and no row that is kept.
 // FW warps share a face: one up to FACE_K1 velocities, two beyond, where the rows of one
 // face per warp (16 bytes x K x 2432 warps) no longer fit L2 until the second pass reads
 // them.  One warp / two warps per face: 0.40 / 0.55 ms at K = 1,517 (53,000 faces), 1.59 /

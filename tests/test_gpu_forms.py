@@ -200,3 +200,28 @@ def test_fp64_scheme_has_the_range_of_fp64(a, b, product):
         z = q / sc
         assert np.abs(z - p).max() <= 1e-10 * np.abs(p).max()
     assert not product or np.isfinite(y[4]).all()
+
+
+def test_mixed_padding_adds_nothing_beside_a_fast_velocity():
+    """126 velocities (two of padding in the last group of four), one of them so fast that
+    the cube of its speed, which the heat-flux terms form, is near the end of FP32's range
+    (its Maxwellian is zero): the fields and macro fluxes are those of the FP64 context to the
+    mixed tolerance."""
+    from paper_2303_10846_gb300.rykov import Solver
+    wl = I.cavity_workload(n=3, n_gh=5)
+    x = wl.mesh.cell_center
+    wl.prim0[:, 0] *= 1.0 + 0.1 * np.sin(5 * x[:, 0] + 3 * x[:, 1])
+    fast = np.array([[2e12, 0.0, 0.0]])
+    for at in (0, 125):
+        u = np.insert(wl.dvs.u, at, fast, axis=0)
+        w = np.insert(wl.dvs.w, at, 1e-3)
+        wl2 = I.Workload(name="fast", mesh=wl.mesh, dvs=I.DVS(u=u, w=w), params=wl.params, bcs=wl.bcs,
+                         prim0=wl.prim0, ref=wl.ref)
+        m, d = Solver(wl2, "mixed"), Solver(wl2, "fp64")
+        for s in (m, d):
+            rc, n, res = s.iterate(2)
+            assert rc == 0 and np.isfinite(res).all()
+        for name in ("W", "MACRO_F"):
+            a, b = m.debug_get(name), d.debug_get(name)
+            assert np.abs(a - b).max() <= 1e-5 * np.abs(b).max(), name
+        assert not m.get_distribution()[:, :, 126:].any()
