@@ -449,15 +449,7 @@ static int bind_impl(rk_ctx* ctx, rk::Dev<T>& d) {
         ctx->sched.maxs = maxs;
         ctx->sched.staged = (ctx->use_staged && rk::Launch<T>::micro_staged_smem(maxs) > 0) ? ctx->use_staged : 0;
         ctx->sched.macro32 = (ctx->prec == RK_MIXED && ctx->use_macro32) ? 1 : 0;
-        // Programmatic serialisation of the macro phases unless RYKOV_PDL says otherwise:
-        // always in mixed contexts (iteration with / without: cavity 12^3 x 343 0.41 / 0.45
-        // ms, sphere 26,928 x 1,517 with the FP32 solve 2.77 / 2.92, cone 75,177 x 7,980
-        // 28.4 / 28.8); in FP64 contexts only while a phase leaves SMs free (cavity 8^3
-        // 1.18 / 1.23), since waiting blocks there hold up the FP64 micro flux beside them
-        // (sphere 37,086 x 304 13.2 / 12.9)
-        const int nmax = *std::max_element(ctx->col_off.begin(), ctx->col_off.end()) / std::max(ctx->C, 1);
-        const bool few = (long long)nmax * rk::macro_lanes(nmax, d.ms) < 152LL * rk::MACRO_BS;
-        ctx->sched.pdl = ctx->use_pdl >= 0 ? ctx->use_pdl : (sizeof(T) == 4 || few);
+        ctx->sched.pdl = ctx->use_pdl >= 0 ? ctx->use_pdl : rk::macro_ahead(ctx->col_off, d.ms, sizeof(T) == 8);
         // RYKOV_MACRO_LANES=1|2|4: threads per cell of the FP32 macro phases, each taking
         // every L-th face (default 4: one face each on tetrahedra)
         if (const char* v = std::getenv("RYKOV_MACRO_LANES")) {

@@ -75,6 +75,18 @@ static inline std::vector<Phase> sgs_phases(const Sched& sc, int n) {
     return ph;
 }
 
+// Whether the macro phases of a context are launched ahead of their turn (programmatic
+// stream serialisation), unless RYKOV_PDL says otherwise: always in mixed contexts
+// (iteration with / without: cavity 12^3 x 343 0.41 / 0.45 ms, sphere 26,928 x 1,517 with the
+// FP32 solve 2.77 / 2.92, cone 75,177 x 7,980 28.4 / 28.8); in FP64 contexts only while the
+// largest phase leaves SMs free (cavity 8^3 x 512 0.65 / 0.71), since waiting blocks hold up
+// the FP64 micro flux beside them (sphere 37,086 x 304 13.6 / 13.2)
+static inline bool macro_ahead(const std::vector<int>& col_off, int ms, bool fp64) {
+    int n = 0;
+    for (size_t c = 0; c + 1 < col_off.size(); ++c) n = std::max(n, col_off[c + 1] - col_off[c]);
+    return !fp64 || (long long)n * macro_lanes(n, ms) < 152LL * MACRO_BS;
+}
+
 // one colour phase, with programmatic stream serialisation if pdl
 template <typename... A, typename... B>
 static inline cudaError_t launch_phase(void (*k)(A...), long long threads, bool pdl, cudaStream_t s, const B&... args) {
