@@ -436,15 +436,18 @@ __global__ void __launch_bounds__(WPB * 32, RECONP_MINB * 8 / WPB)
 // in registers instead the kernel was slower than the scalar form: 9.1 ms against 7.9 on
 // 262,000 faces x 5,991).  No select guards the K padding: it repeats the last velocity with
 // weight zero (see bind_impl), its face values are in no sum and no row that is kept.
-// FW warps share a face: one up to FACE_K1 velocities, two beyond, where the rows of one
-// face per warp (16 bytes x K x 2432 warps) no longer fit L2 until the second pass reads
-// them.  One warp / two warps per face: 0.40 / 0.55 ms at K = 1,517 (53,000 faces), 1.59 /
-// 2.00 at 3,033 (122,000), 8.3 / 7.3 at 5,991 (262,000), 6.5 / 5.4 at 7,980 (150,000);
-// the scalar form took 0.43, 1.89, 7.9 and 6.0 ms.  With reciprocals in the state (one
-// lane's chain): 0.38, 1.55 and 6.85 ms at the first three.
+// FW warps share a face: one up to FACE_K1 velocities, two beyond, where the rows that the
+// faces in flight (2,432 with one warp each, 16 bytes x K) hold between the two passes
+// outgrow L2 (126 MB at K = 3,240, all of it lost by 6,000).  One warp / two warps per face,
+// the kernel and the whole iteration in ms: 61,911 cells, K = 3,033 1.56 / 1.86 and 9.85 /
+// 10.21, 4,096 2.02 / 2.32 and 12.23 / 12.57, 5,000 2.52 / 2.87 and 14.67 / 15.04, 5,991
+// 3.86 / 3.27 and 17.65 / 17.04; 205,504 cells, 4,500 7.40 / 8.59 and 43.1 / 44.5, 5,000 10.9
+// / 9.3 and 47.3 / 48.7, 5,991 12.9 / 11.0 and 54.7 / 55.8 (boundary faces beside it);
+// 131,772 cells, 5,991 8.3 / 7.3; cone 75,177 cells, 7,980 6.5 / 5.4.
+// The scalar form took 0.43 ms at 26,928 x 1,517 (this one 0.38), 1.89 at 61,911 x 3,033.
 // ------------------------------------------------------------------------------------
 constexpr int FACE_ST = 3;
-constexpr int FACE_K1 = 4096;
+constexpr int FACE_K1 = 5120;
 struct Row4 {
     float2 v[2];
 };

@@ -225,3 +225,20 @@ def test_mixed_padding_adds_nothing_beside_a_fast_velocity():
             a, b = m.debug_get(name), d.debug_get(name)
             assert np.abs(a - b).max() <= 1e-5 * np.abs(b).max(), name
         assert not m.get_distribution()[:, :, 126:].any()
+
+
+def test_two_warps_per_interior_face():
+    """5,832 velocities, beyond the line from which two warps share a face (one warp's rows
+    end in the other's range): distributions, fields and face values against the oracle."""
+    import oracle as O
+    from paper_2303_10846_gb300.rykov import Solver
+    wl = I.cavity_workload(n=3, n_gh=18)
+    x = wl.mesh.cell_center
+    wl.prim0[:, 0] *= 1.0 + 0.1 * np.sin(5 * x[:, 0] + 3 * x[:, 1])
+    wl.prim0[:, 4] *= 1.0 + 0.1 * np.cos(4 * x[:, 2])
+    s, o = Solver(wl, "mixed"), O.Oracle(wl)
+    s.iterate(2)
+    o.iterate(2)
+    for name, buf in (("W", O.BUF_W), ("PHI", O.BUF_PHI), ("WT", O.BUF_WT), ("FACE", O.BUF_FACE)):
+        a, b = s.debug_get(name), o.get(buf)
+        assert np.abs(a.ravel() - b.ravel()).max() <= 1e-5 * np.abs(b).max(), name
