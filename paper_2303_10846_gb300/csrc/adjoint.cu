@@ -77,6 +77,11 @@ static size_t adj_carve(rk_ctx* ctx, int m, char* base, AdjState& A) {
     size_t ms = 4;
     for (size_t i = 0; i < N; ++i) ms = std::max<size_t>(ms, ctx->slot_off[i + 1] - ctx->slot_off[i]);
     A.nbg = cv.take<double>(2 * ms * N * Kp);
+    // and, between the products, the preconditioner's temporary and its input at the end of a
+    // restart cycle (4 N K_pad + 12 N doubles of 8 N K_pad at least; each is written in full
+    // before it is read)
+    A.pc1 = A.nbg;
+    A.tmp2 = A.nbg + 2 * N * Kp;
     A.fmom = cv.take<double>((size_t)rk::FMOM * (ctx->Fi + 1));
     A.fsum = cv.take<double>((size_t)(rk::ADJ_FS + 1) * (ctx->Fi + 1));
     A.feq = cv.take<double>((size_t)rk::EQA * (ctx->Fi + 1));
@@ -97,10 +102,8 @@ static size_t adj_carve(rk_ctx* ctx, int m, char* base, AdjState& A) {
     A.lam = cv.take<double>(A.np);
     A.rv = cv.take<double>(A.np);
     A.tmp = cv.take<double>(A.np);
-    A.tmp2 = cv.take<double>(A.np);
     A.V = cv.take<double>((size_t)(m + 1) * A.np);
     A.stage = cv.take<double>(A.n);
-    A.pc1 = cv.take<double>(2 * N * Kp);
     A.pcW = cv.take<double>(12 * N);
     A.mY = cv.take<double>(6 * N);
     A.mYp = cv.take<double>(8 * N);

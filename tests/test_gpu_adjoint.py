@@ -419,3 +419,24 @@ def test_adjoint_product_in_other_units_of_velocity(prec, b):
     st = Steady(base)
     for p, q in zip(_blocks(st, scaled * X), _blocks(st, out)):
         assert _rel(p, q) < (1e-10 if prec == "fp64" else 1e-5)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+@pytest.mark.parametrize("name", ["tet", "lid_farfield"])
+def test_adjoint_workspace_size(name, prec):
+    """In vectors of 2 N K_pad doubles: two face arrays, the neighbours' shares (one a face of
+    a cell) with the preconditioner's two temporaries inside them, five vectors, the staging,
+    the inverse diagonal (1/2), the Krylov space, and of mixed contexts two copies of the
+    state and an FP32 vector; and some 200 doubles a cell of records (faces shared by two)."""
+    import ctypes as C
+    wl = WORKLOADS[name]()
+    s = _solver_prec(wl, prec, 4)
+    m = wl.mesh
+    ms = np.bincount(m.face_cell[m.face_cell >= 0].ravel()).max()
+    for k in (1, 20):
+        n = C.c_size_t()
+        s._check(s.L.rk_adjoint_workspace_size(s.h, k, C.byref(n)))
+        fields = 2 * m.n_face / m.n_cell + ms + 5 + 1 + 0.5 + (k + 1) + (2.5 if prec == "mixed" else 0)
+        records = 60 * ms + 300
+        fixed = 8 * (1024 * 64 + 4096) + 40 * 256
+        assert n.value <= 8 * s.N * (2 * s.Kp * fields + records + 12 * (k + 7)) + fixed
