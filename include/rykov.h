@@ -97,8 +97,9 @@ int rk_version(void);
 /* Create a context of the given precision whose work goes to `cuda_stream`
  * (a cudaStream_t cast to uintptr_t; 0 = legacy default stream).
  * Arithmetic: RK_FP64 computes everything in FP64.  RK_MIXED stores the
- * distributions in FP32 and computes per velocity in FP32, with compensated sums
- * over the velocities combined in FP64, FP64 moments, interface states and
+ * distributions in FP32 and computes per velocity in FP32, interface states from
+ * the moments included, with compensated sums over the velocities carried in
+ * float-float pairs (44 bits) across threads, FP64 moments of the cells and
  * compensation (Step 6), and the macro PR-SGS of Step 4 in FP64.  With the
  * RK_MACRO_FP32 flag the macro PR-SGS runs in FP32 in delta form instead: its
  * constant part is formed in FP64 and every FP32 rounding is relative to the
@@ -110,9 +111,10 @@ int rk_version(void);
  *                       runs out makes rk_implicit_iterate return RK_ETIMEOUT, once);
  *   RYKOV_COOP_UNREACHABLE=1  tests of that bound only: the barriers wait for one
  *                       arrival more than the grid makes, with a 50 ms bound;
- *   RYKOV_STAGED=b      micro sweeps with staged row loads (bit mask, default 4;
- *                       + 8: the cell's own rows by bulk copies with mbarrier
- *                       completion in the packed kernels, same results);
+ *   RYKOV_STAGED=b      RK_MIXED micro sweeps with staged row loads (bit mask, default
+ *                       4; + 8: the cell's own rows by bulk copies with mbarrier
+ *                       completion in the packed kernels, same results; RK_FP64
+ *                       sweeps, bound by arithmetic, have one form);
  *   RYKOV_PRIO=0        no stream priorities in the graph;
  *   RYKOV_PDL=0|1       macro phases without / with programmatic serialisation (default:
  *                       with, except in FP64 contexts whose phases fill the GPU);
@@ -315,8 +317,9 @@ const char* rk_noalloc_last_error(void);
  * Arithmetic: FP64 for RK_FP64 contexts.  RK_MIXED contexts evaluate at their own
  * state (FP32 distributions; rk_put_state rounds phi to FP32) with the per-velocity
  * work of rk_vjp, rk_objective and the GMRES preconditioner in FP32 (velocity sums
- * compensated and combined in FP64; vectors, per-cell and per-face scalars and the
- * Krylov arithmetic in FP64); relative accuracy ~1e-6, except that the limiter's
+ * of four terms at a time compensated, carried in float-float pairs across threads;
+ * vectors, boundary faces, per-cell and per-face scalars and the Krylov arithmetic in
+ * FP64); relative accuracy ~1e-6, except that the limiter's
  * derivative is dropped where the limited differences are below 1e-30 (far tails).
  * The environment variable RYKOV_ADJ_FP64=1 makes mixed contexts use FP64 there too.
  *
