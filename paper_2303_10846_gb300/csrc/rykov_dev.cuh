@@ -28,13 +28,6 @@ constexpr int MAXF = 8;        // faces per cell
 #ifndef FACE_NV
 #define FACE_NV 4            // velocities per lane of k_face_interior in mixed mode (16-byte accesses)
 #endif
-#ifndef FACE_CG
-#define FACE_CG 1            // k_face_interior reads the face rows through L2 only
-#endif
-#ifndef FACE_PADSEL
-#define FACE_PADSEL 1        // 1: the K padding zeroed by a select per velocity (0: in a tail
-                             // branch; measured 43.9 vs 38.6 ms at scale: code generation)
-#endif
 #ifndef MICRO_FLUX_NV
 #define MICRO_FLUX_NV 4
 #endif
@@ -58,14 +51,6 @@ constexpr int MAXF = 8;        // faces per cell
 #endif
 #ifndef MICRO_LAST_PF
 #define MICRO_LAST_PF MICRO_PF
-#endif
-// limiter ratio in mixed mode: 1 = approximate division (__fdividef, 2 ulp)
-#ifndef RECON_FASTDIV
-#define RECON_FASTDIV 1
-#endif
-// mixed-mode limiter: 1 = both evaluations computed and selected without branches
-#ifndef RECON_BF
-#define RECON_BF 1
 #endif
 constexpr int EQN = 24;        // constants of one Rykov equilibrium (see make_eq)
 constexpr int CEQ = 28;        // per-cell record: EQN constants, 1/tau~, diagonal base
@@ -154,12 +139,8 @@ __device__ __forceinline__ double dot_rn(double ax, double ay, double az, double
 __device__ __forceinline__ float dot_rn(float ax, float ay, float az, float bx, float by, float bz) {
     return __fadd_rn(__fadd_rn(__fmul_rn(ax, bx), __fmul_rn(ay, by)), __fmul_rn(az, bz));
 }
-// u.n for the split of the micro operator into diagonal (u.n > 0) and neighbour
-// (u.n < 0) parts: exact-rounded in FP64 (same split as the oracle), contracted in FP32
-__device__ __forceinline__ double dot_split(double ax, double ay, double az, double bx, double by,
-                                            double bz) {
-    return dot_rn(ax, ay, az, bx, by, bz);
-}
+// u.n for the split of the micro operator into diagonal (u.n > 0) and neighbour (u.n < 0)
+// parts, contracted in FP32 (FP64 splits as the oracle: outflow)
 __device__ __forceinline__ float dot_split(float ax, float ay, float az, float bx, float by, float bz) {
     return fmaf(az, bz, fmaf(ay, by, ax * bx));
 }
@@ -259,7 +240,6 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
 // 1/x of a normal x with |x| < 2^1022: the hardware's approximation (rcp.approx.ftz.f64,
 // which takes 20 bits of the mantissa) and one step of Householder's third-order iteration,
 // y (1 + e + e^2) with e = 1 - x y; what is left, e^3 < 2^-57, is below the rounding of the
@@ -273,18 +253,13 @@ __device__ __forceinline__ double inv(double x) {
 }
 __device__ __forceinline__ float inv(float x) { return 1.f / x; }
 __device__ __forceinline__ float rcp(float x) { return __fdividef(1.0f, x); }
-// quotient of the limiter function: exact in FP64 mode
-__device__ __forceinline__ double lim_div(double a, double b) { return a / b; }
+// quotient of the limiter function (FP64 has quot): the approximate division
 __device__ __forceinline__ float lim_div(float a, float b) {
-#if RECON_FASTDIV
     // the approximate quotient takes the reciprocal of b, which overflows for b below
     // ~1e-38 (the distribution tails give such differences): both operands are then
     // scaled by 2^64 first (exact), which leaves the quotient unchanged
     const float sc = b < 1e-30f ? 18446744073709551616.0f : 1.0f;
     return __fdividef(a * sc, b * sc);
-#else
-    return a / b;
-#endif
 }
 
 // Accumulators for sums over the velocity space.  FP64 mode: plain FP64 sum.  Mixed
@@ -368,24 +343,12 @@ struct Red<float> {
     }
 };
 
-template <typename T, int NV>
-__device__ __forceinline__ void warp_red(typename Red<T>::V (&v)[NV]) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[j] = Red<T>::add(v[j], Red<T>::shfl_xor(v[j], o));
-    }
-}
-
 // Sum over the 32 lanes of N values whose totals are needed on lane 0 only
 // (reduce-scatter, then a gather): at the level with lane offset o every lane keeps
 // half of its slots, sending the other half to its partner (one shuffle per kept
 // slot instead of one per value), so the five levels cost ceil(N/2) + ... shuffles
 // and additions instead of 5 N; lane 0 then fetches each total from the lane that
 // holds it.  Fixed order: deterministic.  Other lanes' values are partial sums.
-#ifndef WARP_RED_SCATTER
-#define WARP_RED_SCATTER 1
-#endif
 template <typename T, int NI, int NO>
 __device__ __forceinline__ void red_level(const typename Red<T>::V (&in)[NI], typename Red<T>::V (&out)[NO],
                                           int off) {
@@ -425,15 +388,6 @@ __device__ __forceinline__ void warp_red0(typename Red<T>::V (&v)[N]) {
         v[j] = R::shfl(a5[0], lane);
     }
 }
-template <typename T, int N>
-__device__ __forceinline__ void warp_red_lane0(typename Red<T>::V (&v)[N]) {
-#if WARP_RED_SCATTER
-    warp_red0<T, N>(v);
-#else
-    warp_red<T, N>(v);
-#endif
-}
-
 // Butterfly sum over the 32 lanes of a warp (every lane ends with the same bits).
 template <int NV>
 __device__ __forceinline__ void warp_sum(double (&v)[NV]) {
@@ -511,7 +465,6 @@ __device__ __forceinline__ void vload_cg(const float* p, float (&x)[2]) {
     x[0] = v.x; x[1] = v.y;
 }
 __device__ __forceinline__ void vload_cg(const float* p, float (&x)[1]) { x[0] = __ldcg(p); }
-__device__ __forceinline__ void vload_cg(const double* p, double (&x)[1]) { x[0] = __ldcg(p); }
 __device__ __forceinline__ void vload(const double* p, double (&x)[1]) { x[0] = *p; }
 __device__ __forceinline__ void vload(const float* p, float (&x)[1]) { x[0] = *p; }
 __device__ __forceinline__ void vstore(float* p, const float (&x)[1]) { *p = x[0]; }
@@ -519,14 +472,6 @@ __device__ __forceinline__ void vstore(float* p, const float (&x)[2]) {
     *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
 }
 __device__ __forceinline__ void vstore(double* p, const double (&x)[1]) { *p = x[0]; }
-template <typename T, int NV>
-__device__ __forceinline__ void vload_row(const T* p, T (&x)[NV]) {
-#if FACE_CG
-    vload_cg(p, x);
-#else
-    vload(p, x);
-#endif
-}
 
 // ------------------------------------------------------------------------------------
 // gas model
@@ -796,15 +741,14 @@ struct alignas(4 * sizeof(T)) Q4 {
     T x, y, z, w;
 };
 #ifndef RECON_MINB
-#define RECON_MINB 3         // mixed mode: 80 registers, three blocks of eight warps per SM
-                             // (FP64: four blocks, 64 registers)
+#define RECON_MINB 3         // 80 registers, three blocks of eight warps per SM
 #endif
 // BND: only the cells of the list `cells` and, of their faces, only the boundary ones
 // (all that the wall quantities of a field depend on).
 template <typename T, int WPB, bool BND = false>
-__global__ void __launch_bounds__(WPB * 32, sizeof(T) == 8 ? 4 : RECON_MINB)
+__global__ void __launch_bounds__(WPB * 32, RECON_MINB)
     k_recon(Dev<T> c, const int* cells = nullptr, int ncells = 0) {
-    constexpr int NV = sizeof(T) == 8 ? 1 : RECON_NV;
+    constexpr int NV = RECON_NV;
     __shared__ Q4<T> s_A[WPB][MAXF];              // LSQ weight vector, s_ij
     __shared__ Q4<T> s_B[WPB][MAXF];              // x_f - x_i, s_ij
     __shared__ Q4<T> s_C[WPB][MAXF];              // face normal
@@ -897,32 +841,14 @@ __global__ void __launch_bounds__(WPB * 32, sizeof(T) == 8 ? 4 : RECON_MINB)
                         const T ph0 = fd == 0 ? pg[e] : ph[e];
                         const T ep = eps2 * ph0 * ph0;
                         T Lv = T(1);
-#if RECON_BF
-                        if constexpr (sizeof(T) == 4) {
-                            // the same minimum without branches: both quotients are formed
-                            // (their denominators are positive whenever they are selected)
-                            const T a1 = dmax[fd][e], a2 = d2hi[fd][e];
-                            const T b1 = dmin[fd][e], b2 = d2lo[fd][e];
-                            const T ra = lim_div(a1 * a1 + ep + T(2) * a1 * a2, a1 * a1 + T(2) * a2 * a2 + a1 * a2 + ep);
-                            const T rb = lim_div(b1 * b1 + ep + T(2) * b1 * b2, b1 * b1 + T(2) * b2 * b2 + b1 * b2 + ep);
-                            Lv = (a2 > T(0) && ra < Lv) ? ra : Lv;
-                            Lv = (b2 < T(0) && rb < Lv) ? rb : Lv;
-                            L[fd][e] = Lv;
-                            continue;
-                        }
-#endif
-                        if (d2hi[fd][e] > T(0)) {
-                            const T d1 = dmax[fd][e], d2 = d2hi[fd][e];
-                            const T num = d1 * d1 + ep + T(2) * d1 * d2;
-                            const T den = d1 * d1 + T(2) * d2 * d2 + d1 * d2 + ep;
-                            if (num < den) Lv = lim_div(num, den);
-                        }
-                        if (d2lo[fd][e] < T(0)) {
-                            const T d1 = dmin[fd][e], d2 = d2lo[fd][e];
-                            const T num = d1 * d1 + ep + T(2) * d1 * d2;
-                            const T den = d1 * d1 + T(2) * d2 * d2 + d1 * d2 + ep;
-                            if (num < Lv * den) Lv = lim_div(num, den);
-                        }
+                        // without branches: both quotients are formed (their denominators
+                        // are positive whenever they are selected)
+                        const T a1 = dmax[fd][e], a2 = d2hi[fd][e];
+                        const T b1 = dmin[fd][e], b2 = d2lo[fd][e];
+                        const T ra = lim_div(a1 * a1 + ep + T(2) * a1 * a2, a1 * a1 + T(2) * a2 * a2 + a1 * a2 + ep);
+                        const T rb = lim_div(b1 * b1 + ep + T(2) * b1 * b2, b1 * b1 + T(2) * b2 * b2 + b1 * b2 + ep);
+                        Lv = (a2 > T(0) && ra < Lv) ? ra : Lv;
+                        Lv = (b2 < T(0) && rb < Lv) ? rb : Lv;
                         L[fd][e] = Lv;
                     }
                 if (limiter == 4) {
@@ -1051,7 +977,7 @@ template <typename T, int WPB>
 __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c) {
     using R = Red<T>;
     using V = typename R::V;
-    constexpr int NV = sizeof(T) == 8 ? 1 : FACE_NV;
+    constexpr int NV = FACE_NV;
     constexpr int NB = EQN + 2;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int fi = blockIdx.x * WPB + wib;
@@ -1089,8 +1015,8 @@ __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c)
             vload(c.uT + c.Kp + k0, uy);
             vload(c.uT + 2 * c.Kp + k0, uz);
             vload(c.wT + k0, wv);
-            vload_row(g0 + k0, gv);
-            vload_row(h0 + k0, hv);
+            vload_cg(g0 + k0, gv);
+            vload_cg(h0 + k0, hv);
 #pragma unroll
             for (int e = 0; e < NV; ++e) {
                 const T cx = ux[e] - Ur[0], cy = uy[e] - Ur[1], cz = uz[e] - Ur[2];
@@ -1116,7 +1042,7 @@ __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c)
             v[5 + j] = R::from(t);
         }
     }
-    warp_red_lane0<T, 17>(v);
+    warp_red0<T, 17>(v);
     // interface state on lane 0, in the per-velocity arithmetic type T (the moments
     // themselves are carried with compensation)
     T cst[NB];
@@ -1143,20 +1069,15 @@ __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c)
             vload(c.wT + k0, wv);
 #pragma unroll
             for (int q = 0; q < NV; ++q) u2[q] = T(0.5) * (ux[q] * ux[q] + uy[q] * uy[q] + uz[q] * uz[q]);
-            vload_row(g0 + k0, gv);
-            vload_row(h0 + k0, hv);
+            vload_cg(g0 + k0, gv);
+            vload_cg(h0 + k0, hv);
 #pragma unroll
             for (int q = 0; q < NV; ++q) {
                 T G, H;
                 eval_eq(e + 2, ux[q], uy[q], uz[q], G, H);
-#if FACE_PADSEL
                 const bool pad = k0 + q >= c.K;
                 const T gf = pad ? T(0) : a * gv[q] + b * G;
                 const T hf = pad ? T(0) : a * hv[q] + b * H;
-#else
-                const T gf = a * gv[q] + b * G;
-                const T hf = a * hv[q] + b * H;
-#endif
                 gv[q] = gf;
                 hv[q] = hf;
                 // zero weight in the K padding: no flux terms there
@@ -1166,12 +1087,6 @@ __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c)
 #pragma unroll
                 for (int j = 0; j < 6; ++j) t[j] = q == 0 ? tv[j] : t[j] + tv[j];
             }
-            if (!FACE_PADSEL && k0 + NV > c.K) {
-                // the K padding keeps zero face values
-#pragma unroll
-                for (int q = 0; q < NV; ++q)
-                    if (k0 + q >= c.K) gv[q] = hv[q] = T(0);
-            }
             vstore(g0 + k0, gv);
             vstore(h0 + k0, hv);
 #pragma unroll
@@ -1180,7 +1095,7 @@ __global__ void __launch_bounds__(WPB * 32, FACE_MINB) k_face_interior(Dev<T> c)
 #pragma unroll
         for (int j = 0; j < 6; ++j) r6[j] = R::from(m[j]);
     }
-    warp_red_lane0<T, 6>(r6);
+    warp_red0<T, 6>(r6);
     if (lane == 0)
         for (int d = 0; d < 6; ++d) R::store(c.mface + (size_t)f * 6 + d, r6[d]);
 }
@@ -1248,7 +1163,7 @@ __global__ void __launch_bounds__(BS) k_face_boundary(Dev<T> c, const int* list)
             vstore(g0 + k0, g);
         }
         V v[2] = {R::from(an), R::from(ad)};
-        warp_red_lane0<T, 2>(v);
+        warp_red0<T, 2>(v);
         if (lane == 0) { red[wib][0] = v[0]; red[wib][1] = v[1]; }
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -1293,7 +1208,7 @@ __global__ void __launch_bounds__(BS) k_face_boundary(Dev<T> c, const int* list)
         V v[7];
 #pragma unroll
         for (int j = 0; j < 7; ++j) v[j] = R::from(a[j]);
-        warp_red_lane0<T, 7>(v);
+        warp_red0<T, 7>(v);
         if (lane == 0)
 #pragma unroll
             for (int j = 0; j < 7; ++j) red[wib][j] = v[j];
@@ -2001,7 +1916,7 @@ __global__ void k_macro_finish(Dev<T> c, int m32) {
 template <typename T, int WPB>
 __global__ void __launch_bounds__(WPB * 32) k_micro_flux(Dev<T> c) {
     // velocities per lane: 16-byte accesses in mixed mode
-    constexpr int NV = sizeof(T) == 8 ? 1 : MICRO_FLUX_NV;
+    constexpr int NV = MICRO_FLUX_NV;
     __shared__ int s_face[WPB][MAXF];
     __shared__ T s_n[WPB][3][MAXF], s_AV[WPB][MAXF];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -2130,12 +2045,12 @@ __device__ __forceinline__ void micro_tail(const Dev<T>& c, const T* e, T itau, 
 }
 
 template <typename T, int WPB, bool FIRST, bool LAST>
-__global__ void __launch_bounds__(WPB * 32, sizeof(T) == 8 ? 2 : (LAST ? MICRO_LAST_MINB : (FIRST ? MICRO_FIRST_MINB : MICRO_MID_MINB)))
+__global__ void __launch_bounds__(WPB * 32, LAST ? MICRO_LAST_MINB : (FIRST ? MICRO_FIRST_MINB : MICRO_MID_MINB))
     k_micro_sweep(Dev<T> c, const int* cells, int ncells, int colour) {
     constexpr bool first = FIRST, last = LAST, first_forward = FIRST;
     using R = Red<T>;
     // velocities per lane: 16-byte accesses in the middle sweeps of the mixed mode
-    constexpr int NV = sizeof(T) == 8 ? 1 : (FIRST ? MICRO_FIRST_NV : (LAST ? MICRO_LAST_NV : MICRO_MID_NV));
+    constexpr int NV = FIRST ? MICRO_FIRST_NV : (LAST ? MICRO_LAST_NV : MICRO_MID_NV);
     // faces whose loads are issued together
     constexpr int PF = LAST ? MICRO_LAST_PF : MICRO_PF;
     __shared__ T s_e[WPB][EQN + 2];
@@ -2227,7 +2142,7 @@ __global__ void __launch_bounds__(WPB * 32, sizeof(T) == 8 ? 2 : (LAST ? MICRO_L
         typename R::V v[12];
 #pragma unroll
         for (int j = 0; j < 12; ++j) v[j] = R::from(a[j]);
-        warp_red_lane0<T, 12>(v);
+        warp_red0<T, 12>(v);
         if (lane == 0)
             for (int j = 0; j < 12; ++j) c.S[(size_t)i * 12 + j] = R::to_d(v[j]);
     }
@@ -2260,7 +2175,7 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 #endif
 template <typename T, bool FIRST, bool LAST>
 __host__ __device__ constexpr int micro_nv() {
-    return sizeof(T) == 8 ? 1 : (FIRST ? MICRO_FIRST_NV : (LAST ? MICRO_LAST_NV : MICRO_MID_NV));
+    return FIRST ? MICRO_FIRST_NV : (LAST ? MICRO_LAST_NV : MICRO_MID_NV);
 }
 template <typename T, int WPB, bool FIRST, bool LAST>
 __global__ void __launch_bounds__(WPB * 32)
@@ -2383,7 +2298,7 @@ __global__ void __launch_bounds__(WPB * 32)
         typename R::V v[12];
 #pragma unroll
         for (int j = 0; j < 12; ++j) v[j] = R::from(a[j]);
-        warp_red_lane0<T, 12>(v);
+        warp_red0<T, 12>(v);
         if (lane == 0)
             for (int j = 0; j < 12; ++j) c.S[(size_t)i * 12 + j] = R::to_d(v[j]);
     }

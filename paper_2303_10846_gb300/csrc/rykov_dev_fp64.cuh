@@ -304,7 +304,7 @@ __global__ void __launch_bounds__(WPB * 32, LAST ? 4 : 6)
         }
     }
     if (LAST) {
-        warp_red_lane0<double, 12>(a);
+        warp_red0<double, 12>(a);
         if constexpr (WC > 1) {
             if (lane == 0)
 #pragma unroll
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(WPB * 32) k_face_mom_d(Dev<double> c) {
         m[11] = fma(x, c2, m[11]); m[12] = fma(y, c2, m[12]); m[13] = fma(z, c2, m[13]);
         m[14] = fma(wh, cx, m[14]); m[15] = fma(wh, cy, m[15]); m[16] = fma(wh, cz, m[16]);
     }
-    warp_red_lane0<double, 17>(m);
+    warp_red0<double, 17>(m);
     if (lane == 0) {
         double* o = c.fmom + (size_t)fi * FMOM;
 #pragma unroll
@@ -411,13 +411,13 @@ __global__ void __launch_bounds__(WPB * 32, 8) k_face_flux_d(Dev<double> c) {
         m[4] = fma(wu, fma(c.u2h[k], gf, hf), m[4]);
         m[5] = fma(wu, hf, m[5]);
     }
-    warp_red_lane0<double, 6>(m);
+    warp_red0<double, 6>(m);
     if (lane == 0)
 #pragma unroll
         for (int d = 0; d < 6; ++d) c.mface[(size_t)f * 6 + d] = m[d];
 }
 
-// Warps per block of the FP64 kernels: two, so that the blocks of a small mesh spread
+// Warps per block of the FP64 kernels (the sweeps: four, below): two, so that the blocks of a small mesh spread
 // evenly (an SM's FP64 pipe is the resource: 1,344 faces in blocks of eight warps left some
 // SMs with twice the work of others).  Where there are fewer than FP64_FEW cells (16 warps
 // per SM) the velocities of a cell are split as well, over blocks or, in the sweeps, over

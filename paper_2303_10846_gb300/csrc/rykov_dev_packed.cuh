@@ -535,7 +535,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) k_face_interior_p(Dev<float> c) {
 #pragma unroll
         for (int j = 0; j < 12; ++j) v[5 + j] = ff_of(q[j]);
     }
-    warp_red_lane0<float, 17>(v);
+    warp_red0<float, 17>(v);
     if constexpr (FW > 1) {
         if (lane == 0)
             for (int j = 0; j < 17; ++j) s_v[fib][sub][j] = v[j];
@@ -610,7 +610,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) k_face_interior_p(Dev<float> c) {
 #pragma unroll
         for (int j = 0; j < 6; ++j) r6[j] = Red<float>::from(m[j]);
     }
-    warp_red_lane0<float, 6>(r6);
+    warp_red0<float, 6>(r6);
     if constexpr (FW > 1) {
         if (lane == 0)
             for (int j = 0; j < 6; ++j) s_v[fib][sub][j] = r6[j];
@@ -815,7 +815,7 @@ __global__ void __launch_bounds__(WPB * 32, LAST ? MICROP_LAST_MINB : (FIRST ? M
     if (LAST) {
 #pragma unroll
         for (int j = 0; j < 12; ++j) sums[j] = Red<float>::from(a[j]);
-        warp_red_lane0<float, 12>(sums);
+        warp_red0<float, 12>(sums);
         if (lane == 0)
             for (int j = 0; j < 12; ++j) c.S[(size_t)i * 12 + j] = Red<float>::to_d(sums[j]);
     }
@@ -1071,7 +1071,7 @@ __global__ void __launch_bounds__(WPB * 32)
         FF sums[12];
 #pragma unroll
         for (int j = 0; j < 12; ++j) sums[j] = Red<float>::from(a[j]);
-        warp_red_lane0<float, 12>(sums);
+        warp_red0<float, 12>(sums);
         if (lane == 0)
             for (int j = 0; j < 12; ++j) c.S[(size_t)i * 12 + j] = Red<float>::to_d(sums[j]);
     }
