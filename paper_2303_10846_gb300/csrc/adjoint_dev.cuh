@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(WPB * 32) k_adj_mom(Dev<double> c, AdjBufs a, 
     const S* g0 = r.f0 + (size_t)f * c.Kp;
     const S* h0 = g0 + (size_t)c.F * c.Kp;
     float Ur[3];
-    face_ref_velocity(c, f, lane, Ur);
+    face_ref_velocity<sizeof(S) == 8>(c, f, lane, Ur);
     AdjSum<S, 17> m;
     for (int k0 = NV * lane; k0 < c.K; k0 += 32 * NV) {
         S ux[NV], uy[NV], uz[NV], w[NV], g[NV], h[NV];

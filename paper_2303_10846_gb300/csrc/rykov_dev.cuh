@@ -908,20 +908,25 @@ __global__ void __launch_bounds__(WPB * 32, RECON_MINB)
 #define FACE_MINB 3          // 80 registers, three blocks of eight warps per SM
 #endif
 // Reference velocity U_r of an interior face's moments, the mean of its cells' U^n, on every
-// lane (any value is exact, so it is formed in FP32).  W is first scaled by the power of two
-// of its density, by its exponent bits, so that the range of FP32 is that of U alone, and a
-// velocity beyond it counts as zero.
+// lane (any value is exact, so it is formed in FP32).  WIDE (FP64 moments): W is first scaled
+// by the power of two of its density, by its exponent bits, so that the range of FP32 is that
+// of U alone, and a velocity beyond it counts as zero; FP32 moments have that range
+// themselves, and the scaling costs their kernel 0.25 of 5.4 ms (75,177 cells x 7,980).
+template <bool WIDE>
 __device__ __forceinline__ void face_ref_velocity(const DevBase& c, int f, int lane, float (&Ur)[3]) {
     const double W = lane < 8 ? c.W[6 * (size_t)c.fc[2 * f + (lane >> 2)] + (lane & 3)] : 1.0;
-    const int hi = __double2hiint(W), e = (hi >> 20) & 0x7ff;
-    const int en = e - (((__shfl_sync(0xffffffffu, hi, lane & 4) >> 20) & 0x7ff) - 1023);   // scaled exponent
-    const float wv = e == 0 || en <= 0 ? 0.f
-                                       : (float)__hiloint2double((hi & ~0x7ff00000) | (min(en, 0x7ff) << 20), __double2loint(W));
+    float wv = (float)W;
+    if constexpr (WIDE) {
+        const int hi = __double2hiint(W), e = (hi >> 20) & 0x7ff;
+        const int en = e - (((__shfl_sync(0xffffffffu, hi, lane & 4) >> 20) & 0x7ff) - 1023);   // scaled exponent
+        wv = e == 0 || en <= 0 ? 0.f
+                               : (float)__hiloint2double((hi & ~0x7ff00000) | (min(en, 0x7ff) << 20), __double2loint(W));
+    }
     const float ia = 1.f / __shfl_sync(0xffffffffu, wv, 0), ib = 1.f / __shfl_sync(0xffffffffu, wv, 4);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         const float u = 0.5f * (__shfl_sync(0xffffffffu, wv, 1 + d) * ia + __shfl_sync(0xffffffffu, wv, 5 + d) * ib);
-        Ur[d] = fabsf(u) <= 3.4e38f ? u : 0.f;
+        Ur[d] = !WIDE || fabsf(u) <= 3.4e38f ? u : 0.f;
     }
 }
 // Interface state of Step 2 (b), (c) from the 17 moments x about U_r: the constants e of

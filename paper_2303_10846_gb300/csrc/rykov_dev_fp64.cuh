@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(WPB * 32) k_face_mom_d(Dev<double> c) {
     const double* g0 = c.face + (size_t)f * c.Kp;
     const double* h0 = g0 + (size_t)c.F * c.Kp;
     float Uf[3];
-    face_ref_velocity(c, f, lane, Uf);
+    face_ref_velocity<true>(c, f, lane, Uf);
     const double Ur[3] = {(double)Uf[0], (double)Uf[1], (double)Uf[2]};
     double m[17];
 #pragma unroll

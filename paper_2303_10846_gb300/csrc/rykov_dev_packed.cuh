@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) k_face_interior_p(Dev<float> c) {
         return RowPair{Row4{{lo2(a), hi2(a)}}, Row4{{lo2(b), hi2(b)}}};
     };
     float Ur[3];
-    face_ref_velocity(c, f, lane, Ur);
+    face_ref_velocity<false>(c, f, lane, Ur);
     FF v[17];
     {
         const float2 mx = f2(-Ur[0]), my = f2(-Ur[1]), mz = f2(-Ur[2]);
