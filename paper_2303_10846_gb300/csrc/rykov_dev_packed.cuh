@@ -126,8 +126,9 @@ __device__ __forceinline__ float2 min3_2(float2 a, float2 b, float2 c) {
 #ifndef RECONP_PAIRS
 #define RECONP_PAIRS 3       // bit 0: limiter loop, bit 1: neighbour loop over face pairs
 #endif
-// 1/x in one instruction: without .ftz (and in __fdividef) three or so more rescale the
-// operand near the subnormal range, which the limiter's own scaling keeps away from
+// 1/x by the hardware's approximation (1 ulp), subnormal operands and results flushed to
+// zero: the limiter's own scaling keeps its operands out of that range, which __fdividef
+// allows for (reconstruction of 131,772 x 5,991 with that 7.23 ms, with this 7.04 ms)
 __device__ __forceinline__ float rcp_ftz(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
