@@ -1,8 +1,12 @@
 // Device side of librykov: kernels of one implicit iteration (Sec. 3.5, Steps 2-6)
 // of the conservative implicit Rykov scheme, templated on the storage/arithmetic
 // type T of the per-velocity work (double: FP64 mode; float: mixed mode, where the
-// reductions over the discrete velocity space use compensated FP32 accumulation
-// combined in FP64, and everything per cell or per face stays FP64).
+// reductions over the discrete velocity space use compensated FP32 accumulation carried
+// across threads in float-float pairs, the interface states follow in FP32, and everything
+// per cell stays FP64).  The per-velocity kernels of FP64 contexts are in
+// rykov_dev_fp64.cuh, the packed ones of mixed contexts in rykov_dev_packed.cuh; k_recon,
+// k_face_interior, k_micro_flux and the k_micro_sweep kernels here are the scalar FP32
+// forms (RYKOV_PACKED=0).
 //
 // Layout in HBM (k fastest, K padded to a multiple of 32):
 //   phi, res, dphi : T[2][N][Kp]      face : T[2][F][Kp] (phi(x_ij - u s), then phi_ij)
@@ -149,7 +153,7 @@ __device__ __forceinline__ float dot_split(float ax, float ay, float az, float b
 // the 1e-5 target of the mixed mode)
 __device__ __forceinline__ double ex(double x) { return exp(x); }
 __device__ __forceinline__ float ex(float x) { return __expf(x); }
-// 2^x for the equilibria (exponents pre-scaled by log2(e)): FP64 exp2 in FP64 mode;
+// 2^x for the equilibria (exponents pre-scaled by log2(e)): a table in FP64 mode (below);
 // in mixed mode the hardware approximation (PTX ex2.approx.f32: relative error ~2^-22,
 // subnormal results kept), one instruction where the accurate exp2f takes a longer
 // path for the very negative exponents of the high-speed tails of the DVS
@@ -730,9 +734,8 @@ __global__ void __launch_bounds__(64) k_set_state(Dev<T> c, const double* prim, 
 // ------------------------------------------------------------------------------------
 // Step 2 (a): least-squares gradient, Venkatakrishnan limiter and reconstruction
 // phi(x_ij - u_k s_ij) = phi_c + (x_ij - u_k s_ij - x_c) . L grad phi_c, written by
-// the upwind cell c into the face array (Eq. flux_solve_phi_phi).  One block per
-// cell, velocities strided over the block; the cell's face data staged in shared
-// memory.
+// the upwind cell c into the face array (Eq. flux_solve_phi_phi).  One warp per cell,
+// four velocities per lane; the cell's face data staged in shared memory.
 // ------------------------------------------------------------------------------------
 // per-slot records of the reconstruction, one 16-byte (mixed) or 32-byte (FP64)
 // shared-memory load each
@@ -1968,8 +1971,8 @@ __global__ void __launch_bounds__(WPB * 32) k_micro_flux(Dev<T> c) {
 
 // ------------------------------------------------------------------------------------
 // Step 5 (micro PR-SGS, Eq. implicit_mic_final_equ) and Step 6 (update and integral
-// error compensation, Eqs. solve_rho - solve_qrot).  One block per cell of one
-// colour, velocities strided over the block.
+// error compensation, Eqs. solve_rho - solve_qrot).  One warp per cell of one colour, four
+// velocities per lane.
 //   first sweep : Res = (phi~* - phi^n)/tau~ - F_{i,k}, F from the face array
 //                 (Eq. implicit_mic_flux), stored
 //   every sweep : dphi_i = (Res - sum_j (A/V) min(u.n, 0) dphi_j) / D_{i,k},

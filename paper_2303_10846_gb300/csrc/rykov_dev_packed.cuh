@@ -93,8 +93,8 @@ __global__ void __launch_bounds__(WPB * 32) k_set_eq_p(Dev<float> c) {
 // Two blocks of eight warps per SM (up to 128 registers) with the face loops taken in
 // pairs; 500,949 cells x 7,980: 41.6 ms against 41.9 ms for three blocks with single faces
 // (paired loops spill at three blocks: 43.3 ms; single faces at two blocks: 46.1 ms).
-// Bound by instruction issue (63 %, the ALU pipe of the extremes 47 %) at the 16 warps per
-// SM that the registers leave.  On cells of at most four faces (FOUR) the projections are
+// Bound by instruction issue (59 % of the slots, the ALU pipe of the extremes 42 %; K = 607)
+// at the 16 warps per SM that the registers leave.  On cells of at most four faces (FOUR) the projections are
 // kept and the rows arrive a chunk ahead; 131,772 x 5,991: 8.25 -> 7.23 ms, 61,911 x 3,033
 // 2.03 -> 1.77 ms, 26,928 x 1,517 0.467 -> 0.412 ms (the projections alone 8.18, 2.00 and
 // 0.454 ms: the loads were the larger part); with the bare reciprocal 7.04, 1.72 and
