@@ -344,7 +344,7 @@ const char* rk_noalloc_last_error(void);
  *       iterations done, the final relative residual (recomputed, not estimated),
  *       J, and the total derivative dJdp[6] = dJ/dp + lam^T dR/dp.  RK_EDIVERGED if
  *       the residual becomes non-finite.  The macro operator's spectral radii are the
- *       last iteration's, or those of W where there was none since rk_set_state(_prim).
+ *       last iteration's at the state that it left, and W's at any other state.
  *   rk_adjoint_get(ctx, lam, on_device): the last adjoint solution (packed). */
 /* Fused multiply-add throughput of the current device (a measurement utility with
  * no counterpart in the paper): the ALU ceiling of the FP64 form, whose per-velocity

@@ -402,9 +402,9 @@ static cudaError_t adj_apply(rk_ctx* ctx, AdjState& A, const double* v, double* 
 
 // What the preconditioner needs of the state: the inverse micro diagonal and the constants
 // of the transposed macro updates.  Once per solve.  Its spectral radii are the last
-// iteration's, one step behind the state of a march, or W's where no iteration has formed
-// any since a state was set (they enter the preconditioner alone, so a solve that reaches
-// its tolerance does not depend on them; one that stops at max_iter does).
+// iteration's, one step behind the state that it left, or W's for any other state (they
+// enter the preconditioner alone, so a solve that reaches its tolerance does not depend on
+// them; one that stops at max_iter does).
 template <typename S>
 static cudaError_t adj_pc_prepare_t(rk_ctx* ctx, AdjState& A) {
     const rk::Dev<double> d = dview(ctx, A);
@@ -599,10 +599,23 @@ extern "C" int rk_put_state(rk_ctx* ctx, const double* x, int on_device) {
     CK(cudaGetLastError());
     const rk::DevBase& d = ctx->prec == RK_FP64 ? static_cast<const rk::DevBase&>(ctx->dd)
                                                 : static_cast<const rk::DevBase&>(ctx->df);
+    // the last iteration's radii stay with the state that it left; another W has its own
+    if (ctx->have_radii) {
+        int* differ = reinterpret_cast<int*>(A.hd);
+        CK(cudaMemsetAsync(differ, 0, sizeof(int), ctx->stream));
+        rk::k_adj_differ<<<rk::cdv(6 * N, 256), 256, 0, ctx->stream>>>(src + k1, d.W, 6 * N, differ);
+        CK(cudaGetLastError());
+        CK(cudaMemcpyAsync(A.hpin, differ, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    }
     CK(cudaMemcpyAsync(d.W, src + k1, 6 * N * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemcpyAsync(d.q, src + k1 + 6 * N, 6 * N * sizeof(double), cudaMemcpyDeviceToDevice, ctx->stream));
     CK(cudaMemsetAsync(d.iterp, 0, 4 * sizeof(double), ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
+    if (ctx->have_radii) {
+        int differ = 0;
+        std::memcpy(&differ, A.hpin, sizeof(int));
+        ctx->have_radii = differ == 0;
+    }
     ctx->iter = 0;
     ctx->have_state = true;
     ctx->state_ver++;

@@ -1229,6 +1229,11 @@ __global__ void k_adj_downcast(const double* src, float* dst, size_t n) {
     for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x)
         dst[t] = (float)src[t];
 }
+// *differ = 1 if any of the n doubles of a and b differ in their bits
+__global__ void k_adj_differ(const double* a, const double* b, size_t n, int* differ) {
+    const size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (t < n && __double_as_longlong(a[t]) != __double_as_longlong(b[t])) *differ = 1;
+}
 __global__ void k_adj_slot_s(DevBase c, double* slot_s) {
     const int m = blockIdx.x * blockDim.x + threadIdx.x;
     if (m < c.nnz) slot_s[m] = c.fs[c.slot_face[m]];

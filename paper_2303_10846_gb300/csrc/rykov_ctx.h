@@ -81,8 +81,9 @@ struct rk_ctx {
     // them.  faces_redo: the face step works in place on the reconstruction, so it has to
     // reconstruct first.
     bool faces_partial = false, faces_redo = false;
-    // an iteration (or the flux step) has formed the spectral radii since the workspace was
-    // bound or a state was set by rk_set_state(_prim)
+    // the spectral radii in memory are those of the iteration (or flux step) that led to the
+    // present state: none since the workspace was bound, a state was set by
+    // rk_set_state(_prim), or rk_put_state brought another W
     bool have_radii = false;
     void* dbg = nullptr;                              // [2][N][Kp] T (debug contexts)
     double* pin = nullptr;                            // pinned host: 16 doubles

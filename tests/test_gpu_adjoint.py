@@ -299,17 +299,17 @@ def test_adjoint_sphere_converges_and_matches_finite_differences(sphere_first_or
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
 def test_adjoint_solve_without_an_iteration_before_it(prec):
     """put_state and a bounded solve on a context that never iterated, its workspace full of
-    NaN before the bind, and on one that iterated elsewhere before its state was set: the
-    same bits."""
+    NaN before the bind, and on two that iterated elsewhere (one of them with a state set
+    after that): the same bits."""
     from paper_2303_10846_gb300.rykov import _ptr
     wl = tet()
     donor = _solver_prec(wl, prec, 4)
     donor.iterate(4)
     x = donor.get_state()
     out = []
-    for fresh in (True, False):
+    for before in ("nothing", "another field", "a field set"):
         s = _solver_prec(wl, prec, 4)
-        if fresh:
+        if before == "nothing":
             s.workspace.fill_(255)
             s._check(s.L.rk_bind_workspace(s.h, _ptr(s.workspace), s.workspace.numel()))
             s.bind_adjoint(4)
@@ -319,13 +319,14 @@ def test_adjoint_solve_without_an_iteration_before_it(prec):
             prim[:, 4:6] *= 3.0
             s.set_state_prim(prim)
             s.iterate(3)
-            s.set_state_prim(wl.prim0)
+            if before == "a field set":
+                s.set_state_prim(wl.prim0)
         s.put_state(x)
         it, rel, J, dJdp = s.adjoint_solve("heat", max_iter=6, tol=1e-14)
         assert it == 6 and np.isfinite(rel)
         out.append((s.adjoint_get(), np.array([rel, J]), dJdp))
-    for a, b in zip(*out):
-        assert np.array_equal(a, b)
+    for a, b, c in zip(*out):
+        assert np.array_equal(a, b) and np.array_equal(a, c)
 
 
 def test_mixed_adjoint_at_grazing_velocities(monkeypatch):
