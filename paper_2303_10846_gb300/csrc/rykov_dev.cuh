@@ -433,24 +433,9 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* smem) {
     __syncthreads();
 }
 
-// Per-lane vector width of the velocity loops: two consecutive velocities (8-byte
-// loads) in mixed mode, one in FP64 mode.  Rows are padded to 32 velocities, so the
-// vector accesses never leave a row and stay aligned.
-template <typename T>
-struct VW;
-template <>
-struct VW<float> {
-    static constexpr int N = 2;
-};
-template <>
-struct VW<double> {
-    static constexpr int N = 1;
-};
-__device__ __forceinline__ void vload(const float* p, float (&x)[2]) {
-    const float2 v = *reinterpret_cast<const float2*>(p);
-    x[0] = v.x;
-    x[1] = v.y;
-}
+// Loads and stores of a lane's velocities: four consecutive ones (16 bytes) in FP32, one in
+// FP64.  Rows are padded to 32 velocities, so the vector accesses never leave a row and
+// stay aligned.
 __device__ __forceinline__ void vload(const float* p, float (&x)[4]) {
     const float4 v = *reinterpret_cast<const float4*>(p);
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
@@ -464,17 +449,7 @@ __device__ __forceinline__ void vload_cg(const float* p, float (&x)[4]) {
     const float4 v = __ldcg(reinterpret_cast<const float4*>(p));
     x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
 }
-__device__ __forceinline__ void vload_cg(const float* p, float (&x)[2]) {
-    const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
-    x[0] = v.x; x[1] = v.y;
-}
-__device__ __forceinline__ void vload_cg(const float* p, float (&x)[1]) { x[0] = __ldcg(p); }
 __device__ __forceinline__ void vload(const double* p, double (&x)[1]) { x[0] = *p; }
-__device__ __forceinline__ void vload(const float* p, float (&x)[1]) { x[0] = *p; }
-__device__ __forceinline__ void vstore(float* p, const float (&x)[1]) { *p = x[0]; }
-__device__ __forceinline__ void vstore(float* p, const float (&x)[2]) {
-    *reinterpret_cast<float2*>(p) = make_float2(x[0], x[1]);
-}
 __device__ __forceinline__ void vstore(double* p, const double (&x)[1]) { *p = x[0]; }
 
 // ------------------------------------------------------------------------------------
