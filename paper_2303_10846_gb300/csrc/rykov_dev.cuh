@@ -1437,7 +1437,9 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 // L by macro_lanes: the number of warps that share a sub-partition times the FP64
 // instructions of one warp, which is the phase's time as long as the loads are hidden:
 // per face slot 14, the halving, 20 for the update, or 12 where with eight threads each holds
-// one row of it (INC: 19, 26 and 18, which choose alike).  One thread per cell serves large
+// one row of it (INC: 19, 26 and 18, which choose alike on
+// four to eight faces, but two threads instead of one for 19,457 to 29,184 tetrahedra of a
+// colour: not measured).  One thread per cell serves large
 // colours (no redundant update), more threads the small ones, whose phase is one warp's
 // serial chain: 864 cells with six faces take 8 threads, 32 instructions instead of 104.
 // 40 sweeps with two threads a cell and with this rule, the whole iteration: cavity 12^3 x
